@@ -232,7 +232,8 @@ def kernel_source_hash(kernel: str = "k_hot_batched") -> str:
     """Hash of the code of a neighbourhood kernel (its translation unit and device header,
     comments left out)."""
     h = hashlib.sha256()
-    tu = "psl_alpha2.cu" if kernel.startswith("k_hot_alpha2") else "psl_hot.cu"
+    tu = ("psl_alpha2.cu" if kernel.startswith("k_hot_alpha2") else
+          "psl_lin.cu" if kernel.startswith("k_lin") else "psl_hot.cu")
     for fn in (tu, "psl_device.cuh"):
         with open(os.path.join(ROOT, "paper_2107_09801_gb300", "csrc", fn), encoding="utf-8") as f:
             h.update(_code_only(f.read()).encode())
@@ -242,11 +243,12 @@ def kernel_source_hash(kernel: str = "k_hot_batched") -> str:
 KERNELS_PER_PHASE = {"hot": 1, "select": 1, "recheck": 2, "decide": 1, "apply": 2, "tail": 1}
 
 
-def kernels_per_step(breakdown: dict) -> int:
+def kernels_per_step(breakdown: dict, kernel: str = "") -> int:
     """Kernel launches of one step from a per-phase breakdown of whole steps (a phase's
-    launches count its brackets, one per step)."""
+    launches count its brackets, one per step); `kernel` names the neighbourhood kernels."""
     steps = max(breakdown.get("hot", (0, 0.0))[0], 1)
-    total = sum(KERNELS_PER_PHASE.get(k, 1) * n for k, (n, _) in breakdown.items() if n)
+    per_phase = dict(KERNELS_PER_PHASE, hot=2 if kernel == "k_lin + k_quad" else 1)
+    total = sum(per_phase.get(k, 1) * n for k, (n, _) in breakdown.items() if n)
     return int(round(total / steps))
 
 
@@ -321,13 +323,14 @@ def fp32_error_stats(traces) -> dict:
 def term_counts(L: int) -> dict:
     """Per flip-eval, averaged over the neighbour position j (a window start is uniform):
     nominal terms L-1; live terms (shifts with at least one partner: k <= max(j, L-1-j));
-    and the lookups of the neighbourhood kernel's tables (two per 5 two-partner shifts, one
-    per 5 one-partner shifts)."""
+    and the lookups of the neighbourhood kernel's tables: two per 5 two-partner shifts and one
+    per 5 one-partner shifts, or ("quad") one per 5 two-partner shifts where the rest is a
+    correlation on the tensor cores."""
     j = np.arange(L, dtype=np.float64)
     kin = np.minimum(j, L - 1 - j)
     kout = np.maximum(j, L - 1 - j)
     return {"nominal": float(L - 1), "live": float(kout.mean()),
-            "lookups": float((2.0 * kin / 5.0 + (kout - kin) / 5.0).mean())}
+            "lookups": float((2.0 * kin / 5.0 + (kout - kin) / 5.0).mean()), "quad": float((kin / 5.0).mean())}
 
 
 def measure_alu_peak(local: int, stream) -> dict:
@@ -347,6 +350,8 @@ def hot_roofline(walks_x_N: int, L: int, hot_avg_ms: float, peak: dict, mhz_run:
     measured FP32-add / integer-add / logic-op mix rate, scaled to the clock of the timed region;
     also on live terms, and against the lookup ceiling of the kernel's own inner pattern."""
     tc = term_counts(L)
+    if kernel == "k_lin + k_quad":
+        tc["lookups"] = tc["quad"]
     mhz_peak = peak["clocks"].get("sm_mhz") or peak["max_clock_mhz"]
     scale = (mhz_run / mhz_peak) if (mhz_run and mhz_peak) else 1.0
     p_mix = peak["mix"] * scale
@@ -509,7 +514,7 @@ def run_ours(args):
     # the neighbourhood score, then either the fused tail (short walks) or select, the two
     # re-check kernels (histogram / term sums), decide and the two update passes (ordinary
     # moves; initialisation and switches)
-    launches = args.steps * kernels_per_step(breakdown)
+    launches = args.steps * kernels_per_step(breakdown, hot_name)
 
     # plain form: one walk per launch, one thread per neighbour, host-side selection
     plain = None

@@ -332,10 +332,15 @@ cudaError_t launch_hot_alpha2(const LaunchCtx &c) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_hot(const LaunchCtx &c) { return c.alpha2 ? launch_hot_alpha2(c) : launch_hot_batched(c); }
+cudaError_t launch_hot(const LaunchCtx &c) {
+  if (c.alpha2) return launch_hot_alpha2(c);
+  const cudaError_t e = c.tables ? launch_hot_batched(c) : cudaSuccess;
+  return e == cudaSuccess && c.lin ? launch_hot_lin(c) : e;
+}
 
 int hot_kernel_name(const LaunchCtx &c, char *out, int cap) {
   if (c.alpha2) return snprintf(out, (size_t)cap, "k_hot_alpha2<%u>", c.hot_threads);
+  if (c.lin && !c.tables) return snprintf(out, (size_t)cap, "k_lin + k_quad");
   return hot_batched_name(c, out, cap);
 }
 

@@ -247,6 +247,16 @@ __device__ __forceinline__ float4 tables_for(int c, uint32_t alpha, float inv2e)
   return make_float4((r0 - rb) * S0, (r1 - rb) * S1, (r2 - rb) * S2, (r3 - rb) * S3);
 }
 
+// Scale of the fixed-point coefficients B = (Tm4 - Tp4)/4 and D = (Tm2 - Tp2)/2: both grow with |c|, so
+// their values at the PSL bound them; the result sh keeps |B|, |D| < 2^(35 - sh).
+__device__ __forceinline__ int lin_shift(int psl, uint32_t alpha, int e) {
+  const float4 t = tables_for(psl, alpha, ldexpf(1.f, -e));
+  const float m = fmaxf(0.25f * (fabsf(t.x) + fabsf(t.y)), 0.5f * (fabsf(t.z) + fabsf(t.w))) * 1.0001f;
+  int x;
+  frexpf(m, &x);
+  return 35 - x;
+}
+
 __device__ __forceinline__ float absmax4(float4 t) {
   return fmaxf(fmaxf(fabsf(t.x), fabsf(t.y)), fmaxf(fabsf(t.z), fabsf(t.w)));
 }

@@ -23,6 +23,7 @@ constexpr int kGroupK = 5;         // k per table group (32-entry tables)
 constexpr int kApplyPartStride = 32;  // u32 per apply-chunk partial record
 constexpr int kFlushBlockAdds = 64;   // FP32 additions per lane before a compensated flush
 constexpr int kKsplitMax = 16;        // most k-chunks one neighbour's score may be split into
+constexpr int kLinKsplitMax = 14;     // the same for walks scored by psl_lin.cu (the last two chunks' space holds lin_y)
 constexpr int kKchunkSbUnit = 32;     // k-chunks are whole multiples of 32 super-blocks (960 k)
 constexpr int kWinGuard = 32;         // entries before index 0 and past index L-1 of the partner windows
 
@@ -80,6 +81,7 @@ struct WalkDev {
   uint64_t rng_ctr, moves, flip_evals, switches, rechecks;
   int32_t e;              // table scale exponent: 2^e >= max|C| + 4 over the next window
   float S_abs;            // sum_k max |T_k| (bounds the FP32 error of every score)
+  int32_t lin_sh;         // fixed-point coefficients of psl_lin.cu are multiples of 2^-lin_sh, below 2^35 of them
   uint32_t nktau, ktau_on;
   int32_t ktau_thr;       // list threshold on |C_k| for the running update pass
   uint32_t ncand;
@@ -90,7 +92,8 @@ struct WalkDev {
   uint32_t arrive;
   uint32_t alpha_next;
   uint32_t ksplit, kchunk_sb;  // k-chunks of the neighbourhood kernel and their size (super-blocks)
-  uint32_t kc_psl, pad_kc;     // the k-chunk whose blocks also compute the neighbours' exact PSL
+  uint32_t kc_psl;             // the k-chunk whose blocks also compute the neighbours' exact PSL
+  uint32_t lin;                // scored by psl_lin.cu (its own error bound)
   uint32_t inject_stall;       // test hook: the next neighbourhood pass waits on copies never issued
   float score_min, bound;
   uint32_t flips[kMaxFlips];
@@ -114,11 +117,12 @@ struct Schedule {
   uint32_t max_chunk_apply;  // most update-pass chunks of any listed walk
   uint32_t max_chunk_rc;     // most re-check chunks of any listed walk
   uint32_t hot_next;         // next neighbourhood item to hand out (reset by k_decide)
+  uint32_t quad_next;        // the same for k_quad
   uint32_t general;          // some listed walk needs the general update pass (initialisation or a phase
                              // switch): set by the host and by k_decide, cleared by k_select
   uint32_t alpha2;           // the batch is scored by the alpha = 2 closed form: every neighbour's exact
                              // Delta F is in its walk's score_part (as int32), so the re-check copies it
-  uint32_t pad;
+  uint32_t nquad, nlin;      // work items of k_quad and k_lin, listed after the nitems others in this order
 };
 
 struct LaunchCtx {
@@ -131,6 +135,8 @@ struct LaunchCtx {
   uint32_t hot_flush_sb;   // super-blocks per block sum of the batched kernel (4 or 8)
   uint32_t sm_count;
   uint32_t alpha2;         // every running walk has alpha = 2 and L <= kA2MaxL: the closed-form score
+  uint32_t lin;            // some walk is scored by psl_lin.cu
+  uint32_t tables;         // some walk is scored by the tables of psl_hot.cu (or the closed form)
   uint32_t maxL;           // longest walk of an initialisation launch
   uint32_t ninit;          // walks of an initialisation launch
   cudaStream_t stream;
@@ -154,6 +160,8 @@ cudaError_t prepare_alpha2_kernels();
 // snprintf-style: the length of the full name
 int hot_kernel_name(const LaunchCtx &c, char *out, int cap);
 int hot_batched_name(const LaunchCtx &c, char *out, int cap);
+cudaError_t launch_hot_lin(const LaunchCtx &c);  // psl_lin.cu
+cudaError_t prepare_lin_kernels();
 cudaError_t launch_hot_plain(WalkDev *hdr_one, uint32_t N, cudaStream_t s);
 cudaError_t launch_select(const LaunchCtx &c);
 cudaError_t launch_recheck(const LaunchCtx &c);
@@ -162,6 +170,16 @@ cudaError_t launch_step_tail(const LaunchCtx &c);  // select..apply in one kerne
 constexpr uint32_t kA2MaxL = 4095;  // walks up to this length can take the alpha = 2 closed form
 constexpr uint32_t kA2PerThread = 4;  // window positions per thread of the closed-form kernel (per work item:
                                       // this many times the block size)
+constexpr uint32_t kLinTilePos = 8192;   // window positions per k_lin tile
+// Walks that psl_lin.cu scores faster than the tables: it saves lookups in proportion to N L and costs a
+// tile's chunks, about L + 20000 positions each (partners, and the rows that the tile's ends add).
+// 1024 walks with N = 6912, milliseconds a step, tables / psl_lin.cu: L = 16384 4.98 / 5.02, 18001 5.43 / 5.25,
+// 20001 5.94 / 5.44, 24577 7.18 / 5.94, 32767 9.29 / 6.81, 131071 38.3 / 21.2.
+inline bool lin_pays(uint32_t L, uint32_t N) {
+  const uint64_t tiles = (N + kLinTilePos - 1) / kLinTilePos;
+  return (uint64_t)N * L >= 3300ull * ((uint64_t)L + 20000u) * tiles;
+}
+constexpr uint32_t kQuadPos = 448;       // window positions per k_quad item
 constexpr uint32_t kTailMaxL = kApplyChunk;      // walks up to this length (one update chunk, one re-check chunk)
 constexpr uint32_t kTailMaxN = 2048;             // and windows up to this size (one warp selects)
 cudaError_t launch_start_init(const LaunchCtx &c);
@@ -179,6 +197,18 @@ __host__ __device__ inline double score_bound(float S_abs, uint32_t alpha, uint3
   const double nflush = (double)(L / kSbK + 2 * ksplit);
   const double rel = (2.0 * alpha + 68.0 + 2.0 * ksplit) * u + (nflush * u) * (nflush * u);
   return rel * (double)S_abs * 1.01 + (double)L * 7.52316384526264e-37;  // + L * 2^-120
+}
+
+// Additional error of a score of psl_lin.cu: two units of 2^-lin_sh per shift (each coefficient is a
+// difference of two roundings), and at most 24 more roundings of a partial sum (the boundary
+// terms, flushed every 16, and the correlation's sum joining the tables').
+__host__ __device__ inline double lin_bound(float S_abs, uint32_t L, double unit) {
+  return 24.0 * 5.9604644775390625e-08 * (double)S_abs * 1.01 + 2.0 * (double)L * unit;
+}
+
+// k_lin's sums (fixed point), in the space of the k-chunks above kLinKsplitMax
+__device__ __forceinline__ long long *lin_y(const WalkDev &W) {
+  return reinterpret_cast<long long *>(W.score_part + (size_t)kLinKsplitMax * W.N);
 }
 
 }  // namespace psl

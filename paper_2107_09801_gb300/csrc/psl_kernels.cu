@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(1024) k_select(WalkDev *hdr, const uint32_t *a
 
 __global__ void __launch_bounds__(256) k_decide(WalkDev *hdr, const uint32_t *active, Schedule *sched) {
   // the neighbourhood kernel of this step has finished: rearm its work counter
-  if (blockIdx.x == 0 && threadIdx.x == 0) sched->hot_next = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) sched->hot_next = sched->quad_next = 0;
   for (uint32_t a = blockIdx.x; a < sched->nactive; a += gridDim.x) {
     __syncthreads();
     WalkDev &W = hdr[active[a]];
@@ -222,6 +222,7 @@ static cudaError_t prepare_kernels_once() {
   if (e0 != cudaSuccess) return e0;
   e0 = prepare_hot_kernels();
   if (e0 == cudaSuccess) e0 = prepare_alpha2_kernels();
+  if (e0 == cudaSuccess) e0 = prepare_lin_kernels();
   if (e0 == cudaSuccess) e0 = prepare_recheck_kernel();
   if (e0 == cudaSuccess) e0 = prepare_tail_kernel();
   if (e0 != cudaSuccess) return e0;

@@ -150,6 +150,8 @@ struct psl_ctx {
   int64_t next_id = 0;
   uint32_t hot_flush_sb = 8;  // super-blocks per block sum of the neighbourhood kernel
   bool tail_fused = false;    // every running walk is short: select..apply run as one kernel
+  bool lin = false;           // some running walk is long: scored by psl_lin.cu
+  bool tables = false;        // some running walk is not
   bool alpha2 = false;        // every running walk has alpha1 = alpha2 = 2, L <= kA2MaxL: closed-form score
   uint32_t sm_count = 152;   // SMs the persistent kernels are sized for
   uint32_t dev_sms = 152;    // SMs of the device
@@ -579,7 +581,29 @@ static int rebuild_active(psl_ctx *ctx) {
   ctx->max_chunk_rc = 1;
   // short walks run their few super-blocks with shorter block sums (less unrolled code)
   uint32_t maxL = 0;
-  for (uint32_t s : ctx->active) maxL = std::max(maxL, ctx->h_hdr[s].L);
+  // Long walks are scored by psl_lin.cu when their tiles fill at least half the SMs, all others by the
+  // tables of psl_hot.cu.  Milliseconds a step, tables / psl_lin.cu: 76 walks of L = 131071 2.75 / 1.84, of
+  // L = 32767 0.76 / 0.69; one walk of L = 131071 (split over the SMs) 0.13 / 0.20.
+  uint64_t tiles = 0;
+  for (uint32_t s : ctx->active)
+    if (lin_pays(ctx->h_hdr[s].L, ctx->h_hdr[s].N)) tiles += (ctx->h_hdr[s].N + kLinTilePos - 1) / kLinTilePos;
+  const bool use_lin = ctx->cfg.form == PSL_FORM_BATCHED && 2 * tiles >= ctx->sm_count;
+  bool any_lin = false, any_tab = false;
+  for (uint32_t s : ctx->active) {
+    WalkDev &h = ctx->h_hdr[s];
+    const uint32_t was = h.lin;
+    h.lin = use_lin && lin_pays(h.L, h.N) && h.shard_count <= 1 ? 1u : 0u;
+    if (h.lin && !was && h.moves > 0)  // the space of lin_y may hold partial scores of the tables
+      CK(cudaMemsetAsync(h.score_part + (size_t)kLinKsplitMax * h.N, 0, 8 * (size_t)h.N, ctx->stream));
+    if (!h.lin) maxL = std::max(maxL, h.L);
+    any_lin = any_lin || h.lin;
+    any_tab = any_tab || !h.lin;
+  }
+  if (any_lin != ctx->lin || any_tab != ctx->tables) {
+    ctx->lin = any_lin;
+    ctx->tables = any_tab;
+    drop_graph(ctx);  // captured with other kernels
+  }
   const uint32_t fb = hot_flush_for(maxL);
   if (fb != ctx->hot_flush_sb) {
     ctx->hot_flush_sb = fb;
@@ -606,21 +630,27 @@ static int rebuild_active(psl_ctx *ctx) {
   }
   // Split every walk's k range into chunks when the neighbour blocks alone would leave
   // SMs idle (few walks, or a long walk on its own): aim for about four blocks per SM.
-  const uint32_t T_ = (uint32_t)ctx->cfg.hot_threads * (a2 ? kA2PerThread : 1u);  // window positions per item
+  const uint32_t T_tab = (uint32_t)ctx->cfg.hot_threads * (a2 ? kA2PerThread : 1u);  // window positions per item
+  std::vector<HotItem> quad;
   uint64_t nblocks = 0;
-  for (uint32_t s : ctx->active) nblocks += (ctx->h_hdr[s].N + T_ - 1) / T_;
+  for (uint32_t s : ctx->active) {
+    const uint32_t T_ = ctx->h_hdr[s].lin ? kQuadPos : T_tab;
+    nblocks += (ctx->h_hdr[s].N + T_ - 1) / T_;
+  }
   const uint64_t target = 4ull * (uint64_t)ctx->sm_count;
   uint32_t want = nblocks == 0 ? 1u : (uint32_t)std::min<uint64_t>(kKsplitMax, (target + nblocks - 1) / nblocks);
   if (ctx->cfg.form == PSL_FORM_PLAIN || a2) want = 1;  // these kernels score each neighbour whole
   for (uint32_t s : ctx->active) {
     WalkDev &h = ctx->h_hdr[s];
     const uint32_t unitK = kKchunkSbUnit * kSbK;
-    const uint32_t max_split = std::max<uint32_t>(1u, (h.L - 1 + unitK - 1) / unitK);
-    uint32_t ks = std::min(want, max_split);
+    const uint32_t T_ = h.lin ? kQuadPos : T_tab;
+    const uint32_t span = h.lin ? h.L / 2 : h.L - 1;  // shifts to split: psl_lin.cu looks up k <= kin < L/2 only
+    const uint32_t max_split = std::max<uint32_t>(1u, (span + unitK - 1) / unitK);
+    uint32_t ks = std::min({want, max_split, (uint32_t)(h.lin ? kLinKsplitMax : kKsplitMax)});
     const uint32_t R = h.shard_count;
     if (R > 1)  // a sharded walk: the same chunks on every rank whatever its SM count, the same number per rank
       ks = std::min<uint32_t>(kKsplitMax, max_split) / R * R;
-    const uint32_t units = ((h.L - 1 + unitK - 1) / unitK + ks - 1) / ks;  // chunk size in 960-k units
+    const uint32_t units = ((span + unitK - 1) / unitK + ks - 1) / ks;  // chunk size in 960-k units
     h.ksplit = ks;
     h.kchunk_sb = units * kKchunkSbUnit;
     h.kc_psl = R > 1 ? h.shard_rank : 0u;  // the rank's first chunk also computes the neighbours' PSL
@@ -628,9 +658,28 @@ static int rebuild_active(psl_ctx *ctx) {
     CK(xfer(ctx, (char *)(ctx->d_hdr + s) + offsetof(WalkDev, ksplit), &h.ksplit, 16, cudaMemcpyHostToDevice));
     for (uint32_t i0 = 1; i0 <= h.N; i0 += T_)
       for (uint32_t c = 0; c < ks; c++)
-        if (R <= 1 || c % R == h.shard_rank) items.push_back(HotItem{s, i0, c, 0});
+        if (R <= 1 || c % R == h.shard_rank) (h.lin ? quad : items).push_back(HotItem{s, i0, c, 0});
     ctx->max_chunk_apply = std::max(ctx->max_chunk_apply, h.nchunk_apply);
     ctx->max_chunk_rc = std::max(ctx->max_chunk_rc, h.nchunk_rc);
+  }
+  // k_lin's items: the tiles of every walk (one more where the window may wrap around the end), each
+  // walk's partners split over several items when the tiles alone would leave SMs idle
+  const size_t nitems = items.size(), nquad = quad.size();
+  items.insert(items.end(), quad.begin(), quad.end());
+  if (any_lin) {
+    const uint32_t split = (uint32_t)std::max<uint64_t>(1, ctx->sm_count / tiles);
+    // tile 0 of every walk first: most windows end there, and the blocks take the items in turn
+    bool more = true;
+    for (uint32_t t = 0; more; t++) {
+      more = false;
+      for (uint32_t s : ctx->active) {
+        const WalkDev &h = ctx->h_hdr[s];
+        if (!h.lin) continue;
+        const uint32_t nt = (h.N + kLinTilePos - 1) / kLinTilePos + (h.N < h.L ? 1u : 0u);
+        more = more || t + 1 < nt;
+        for (uint32_t c = 0; t < nt && c < split; c++) items.push_back(HotItem{s, t, c, split});
+      }
+    }
   }
   if (items.size() > ctx->items_cap) {
     CK(cudaStreamSynchronize(ctx->stream));
@@ -639,7 +688,7 @@ static int rebuild_active(psl_ctx *ctx) {
     CK(cudaMalloc(&ctx->d_items, sizeof(HotItem) * ctx->items_cap));
     drop_graph(ctx);  // the captured steps point at the old buffer
   }
-  ctx->nitems = (uint32_t)items.size();
+  ctx->nitems = (uint32_t)nitems;
   if (!items.empty())
     CK(xfer(ctx, ctx->d_items, items.data(), sizeof(HotItem) * items.size(), cudaMemcpyHostToDevice));
   if (!ctx->active.empty()) {
@@ -649,6 +698,8 @@ static int rebuild_active(psl_ctx *ctx) {
   Schedule sc{};
   sc.nactive = (uint32_t)ctx->active.size();
   sc.nitems = ctx->nitems;
+  sc.nquad = (uint32_t)nquad;
+  sc.nlin = (uint32_t)(items.size() - nitems - nquad);
   sc.max_chunk_apply = ctx->max_chunk_apply;
   sc.max_chunk_rc = ctx->max_chunk_rc;
   sc.hot_next = 0;
@@ -670,6 +721,8 @@ static LaunchCtx launch_ctx(psl_ctx *ctx, const uint32_t *d_list, Schedule *d_sc
   c.hot_tile_sb = (uint32_t)ctx->cfg.hot_tile_sb;
   c.hot_flush_sb = ctx->hot_flush_sb;
   c.alpha2 = ctx->alpha2 ? 1u : 0u;
+  c.lin = ctx->lin ? 1u : 0u;
+  c.tables = ctx->tables ? 1u : 0u;
   c.sm_count = ctx->sm_count;
   c.stream = ctx->stream;
   return c;
@@ -1283,6 +1336,7 @@ extern "C" int psl_autotune(psl_ctx *ctx, int reps) {
   if (rc) return rc;
   if (ctx->active_dirty && (rc = rebuild_active(ctx))) return rc;
   if (ctx->active.empty()) return fail(ctx, PSL_ESTATE, "no running walk to tune on");
+  if (!ctx->tables) return ctx->cfg.hot_threads | (ctx->cfg.hot_tile_sb << 16);  // one configuration
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
   CK(cudaEventCreate(&b));
@@ -1297,13 +1351,13 @@ extern "C" int psl_autotune(psl_ctx *ctx, int reps) {
       ctx->cfg.hot_tile_sb = sb;
       if ((rc = rebuild_active(ctx))) return rc;
       LaunchCtx c = launch_ctx(ctx, ctx->d_active, ctx->d_sched);
-      uint32_t *next = &ctx->d_sched->hot_next;
+      uint32_t *next = &ctx->d_sched->hot_next;  // and quad_next after it
       CK(launch_hot(c));  // warm-up
-      CK(cudaMemsetAsync(next, 0, 4, ctx->stream));
+      CK(cudaMemsetAsync(next, 0, 8, ctx->stream));
       CK(cudaEventRecord(a, ctx->stream));
       for (int r = 0; r < reps; r++) {
         CK(launch_hot(c));
-        CK(cudaMemsetAsync(next, 0, 4, ctx->stream));  // the persistent kernel consumed its work counter
+        CK(cudaMemsetAsync(next, 0, 8, ctx->stream));  // the persistent kernel consumed its work counter
       }
       CK(cudaEventRecord(b, ctx->stream));
       CK(cudaEventSynchronize(b));

@@ -120,8 +120,11 @@ __device__ __forceinline__ void apply_finish(WalkDev &W, uint32_t chunk, uint32_
   }
   if (keep_local)
     for (int w = threadIdx.x; w < nw; w += blockDim.x) W.bits_local[w] = W.bits[w];
-  if (mode == kModeInit)
+  if (mode == kModeInit) {
     for (int w = threadIdx.x; w < nw; w += blockDim.x) W.bits_best[w] = W.bits[w];
+    long long *Y = lin_y(W);  // every score pass adds to zeros and leaves zeros
+    for (int i = threadIdx.x; i < (int)W.N; i += blockDim.x) Y[i] = 0;
+  }
   if (threadIdx.x == 0) {
     int m = 0;
     float s = 0.f;
@@ -145,6 +148,7 @@ __device__ __forceinline__ void apply_finish(WalkDev &W, uint32_t chunk, uint32_
     }
     W.psl = m;
     W.S_abs = s;
+    W.lin_sh = lin_shift(m, alpha, W.e);
     W.alpha = alpha;
     if (need_F) {
       wide_store(W.F, Fs);
@@ -378,7 +382,7 @@ __device__ __forceinline__ void select_one(WalkDev &W) {
   }
   __syncthreads();
   m = s_m;
-  const double B = score_bound(W.S_abs, W.alpha, W.L, ksplit);
+  const double B = score_bound(W.S_abs, W.alpha, W.L, ksplit) + (W.lin ? lin_bound(W.S_abs, W.L, scalbn(1.0, -W.lin_sh)) : 0.0);
   const float thr = __double2float_ru((double)m + 2.0 * B);
 
   // ordered compaction of {i : score <= thr}: each thread owns a contiguous segment
@@ -505,7 +509,7 @@ __device__ __forceinline__ void select_warp(WalkDev &W) {
   for (int i = lane; i < N; i += 32) m = fminf(m, score[i]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const double B = score_bound(W.S_abs, W.alpha, W.L, ksplit);
+  const double B = score_bound(W.S_abs, W.alpha, W.L, ksplit) + (W.lin ? lin_bound(W.S_abs, W.L, scalbn(1.0, -W.lin_sh)) : 0.0);
   const float thr = __double2float_ru((double)m + 2.0 * B);
 
   // ordered compaction of {i : score <= thr}
