@@ -172,42 +172,47 @@ __device__ __forceinline__ void group_generic(float &a0, float &a1, uint32_t bsw
   }
 }
 
+// The partner windows are read two positions early, so that a super-block's 30 bits start at bit 2 and
+// field q of a word is a table's byte offset after one shift by 5 q; sums go in pairs (add.f32x2).
+// (The loop is bound by issue and ALU slots.  256 walks of L = 4093 switching phase: 131.4 -> 127.5 ms for 200
+// steps; 64 walks of L = 8191 from their starts: 36.7 -> 35.5 ms; one walk of L = 131071: 26.6 -> 25.8 ms.)
+template <int Q>
+__device__ __forceinline__ uint32_t field4w(uint32_t w) {
+  return (w >> (5 * Q)) & 0x7Cu;
+}
+template <int OFF0, int OFF1>
+__device__ __forceinline__ void add2(float2 &a, uint32_t addr0, uint32_t addr1) {
+  const float v0 = lds_at<OFF0>(addr0), v1 = lds_at<OFF1>(addr1);
+  a = __fadd2_rn(a, make_float2(v0, v1));
+}
+
 // One super-block where every lane has both partners for all 30 shifts; wu and wv point at
-// the lane's forward and backward partner windows of the super-block's first shift.
+// the lane's forward and backward partner windows of the super-block's first shift, two positions early.
 template <bool MB>
-__device__ __forceinline__ void sb_interior(float &a0, float &a1, const uint32_t *__restrict__ wu,
-                                            const uint32_t *__restrict__ wv, uint32_t M, uint32_t bsw) {
+__device__ __forceinline__ void sb_interior(float2 &a, const uint32_t *__restrict__ wu, const uint32_t *__restrict__ wv,
+                                            uint32_t M, uint32_t bsw) {
   constexpr int GS = TabLayout<MB>::GS;
   const uint32_t U = __ldg(wu);
   const uint32_t V = __ldg(wv);
   const uint32_t W1 = (U ^ M) & (V ^ M), W0 = ~((U ^ M) | (V ^ M));
-  a0 += lds_at<0 * GS>(field4<0>(W1) ^ bsw);
-  a1 += lds_at<0 * GS + 128>(field4<0>(W0) ^ bsw);
-  a0 += lds_at<1 * GS>(field4<1>(W1) ^ bsw);
-  a1 += lds_at<1 * GS + 128>(field4<1>(W0) ^ bsw);
-  a0 += lds_at<2 * GS>(field4<2>(W1) ^ bsw);
-  a1 += lds_at<2 * GS + 128>(field4<2>(W0) ^ bsw);
-  a0 += lds_at<3 * GS>(field4<3>(W1) ^ bsw);
-  a1 += lds_at<3 * GS + 128>(field4<3>(W0) ^ bsw);
-  a0 += lds_at<4 * GS>(field4<4>(W1) ^ bsw);
-  a1 += lds_at<4 * GS + 128>(field4<4>(W0) ^ bsw);
-  a0 += lds_at<5 * GS>(field4<5>(W1) ^ bsw);
-  a1 += lds_at<5 * GS + 128>(field4<5>(W0) ^ bsw);
+  add2<0 * GS, 0 * GS + 128>(a, field4w<0>(W1) ^ bsw, field4w<0>(W0) ^ bsw);
+  add2<1 * GS, 1 * GS + 128>(a, field4w<1>(W1) ^ bsw, field4w<1>(W0) ^ bsw);
+  add2<2 * GS, 2 * GS + 128>(a, field4w<2>(W1) ^ bsw, field4w<2>(W0) ^ bsw);
+  add2<3 * GS, 3 * GS + 128>(a, field4w<3>(W1) ^ bsw, field4w<3>(W0) ^ bsw);
+  add2<4 * GS, 4 * GS + 128>(a, field4w<4>(W1) ^ bsw, field4w<4>(W0) ^ bsw);
+  add2<5 * GS, 5 * GS + 128>(a, field4w<5>(W1) ^ bsw, field4w<5>(W0) ^ bsw);
 }
 
 // One super-block where every lane has exactly one partner for all 30 shifts; we points at
-// the lane's window of that partner (forward or backward) for the super-block's first shift.
+// the lane's window of that partner (forward or backward) for the super-block's first shift, two
+// positions early.
 template <bool MB>
-__device__ __forceinline__ void sb_edge(float &a0, float &a1, const uint32_t *__restrict__ we, uint32_t M,
-                                        uint32_t bsw) {
+__device__ __forceinline__ void sb_edge(float2 &a, const uint32_t *__restrict__ we, uint32_t M, uint32_t bsw) {
   constexpr int GS = TabLayout<MB>::GS;
   const uint32_t E = __ldg(we) ^ M;
-  a0 += lds_at<0 * GS + 256>(field4<0>(E) ^ bsw);
-  a1 += lds_at<1 * GS + 256>(field4<1>(E) ^ bsw);
-  a0 += lds_at<2 * GS + 256>(field4<2>(E) ^ bsw);
-  a1 += lds_at<3 * GS + 256>(field4<3>(E) ^ bsw);
-  a0 += lds_at<4 * GS + 256>(field4<4>(E) ^ bsw);
-  a1 += lds_at<5 * GS + 256>(field4<5>(E) ^ bsw);
+  add2<0 * GS + 256, 1 * GS + 256>(a, field4w<0>(E) ^ bsw, field4w<1>(E) ^ bsw);
+  add2<2 * GS + 256, 3 * GS + 256>(a, field4w<2>(E) ^ bsw, field4w<3>(E) ^ bsw);
+  add2<4 * GS + 256, 5 * GS + 256>(a, field4w<4>(E) ^ bsw, field4w<5>(E) ^ bsw);
 }
 
 // One super-block where region boundaries fall inside it for some lane of the warp.
@@ -376,7 +381,8 @@ __device__ __forceinline__ bool hot_one(WalkDev *hdr, const HotItem *items, Sche
     if (threadIdx.x == 0) take_next(true, pipe.seq);
   }
 
-  float hi = 0.f, lo = 0.f, a0 = 0.f, a1 = 0.f;
+  float hi = 0.f, lo = 0.f;
+  float2 a = make_float2(0.f, 0.f);
   for (int tile = 0; tile < ntiles; tile++) {
     const int kt0 = 1 + (tile_lo + tile) * kTileK;
     const uint32_t cq = pipe.seq + (uint32_t)tile;  // this tile's copy
@@ -420,52 +426,52 @@ __device__ __forceinline__ bool hot_one(WalkDev *hdr, const HotItem *items, Sche
     const uint32_t bsw0 = tab_s;  // super-block sb: base + SBB sb, swizzle sb << 2
     int sb = 0;
     {
-      const uint32_t *wu = win_f + (j + kt0), *wv = win_r + (j - kt0);
+      const uint32_t *wu = win_f + (j + kt0 - 2), *wv = win_r + (j - kt0 + 2);
       uint32_t bsw = bsw0;
       // FB super-blocks per flush: at most 6 FB additions into either accumulator
       for (; sb + FB - 1 < n_int; sb += FB) {
 #pragma unroll
-        for (int u = 0; u < FB; u++) sb_interior<MB>(a0, a1, wu + u * kSbK, wv - u * kSbK, M, bsw + u * (SBB + 4));
-        flush2(hi, lo, a0, a1);
+        for (int u = 0; u < FB; u++) sb_interior<MB>(a, wu + u * kSbK, wv - u * kSbK, M, bsw + u * (SBB + 4));
+        flush2(hi, lo, a.x, a.y);
         wu += FB * kSbK, wv -= FB * kSbK, bsw += FB * (SBB + 4);
       }
       if (sb < n_int) {
         for (; sb < n_int; sb++) {
-          sb_interior<MB>(a0, a1, wu, wv, M, bsw);
+          sb_interior<MB>(a, wu, wv, M, bsw);
           wu += kSbK, wv -= kSbK, bsw += SBB + 4;
         }
-        flush2(hi, lo, a0, a1);
+        flush2(hi, lo, a.x, a.y);
       }
     }
     const float4 *Ts = stage + (cq & 1u) * kTileK;  // this tile's per-k values, still staged
     for (; sb < e0; sb++) {
-      sb_generic<MB>(a0, a1, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
+      sb_generic<MB>(a.x, a.y, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
                      bsw0 + sb * (SBB + 4), L, wr);
-      flush2(hi, lo, a0, a1);
+      flush2(hi, lo, a.x, a.y);
     }
     {
       const int step = plus_side ? kSbK : -kSbK;
-      const uint32_t *we = plus_side ? win_f + (j + kt0 + sb * kSbK) : win_r + (j - kt0 - sb * kSbK);
+      const uint32_t *we = plus_side ? win_f + (j + kt0 + sb * kSbK - 2) : win_r + (j - kt0 - sb * kSbK + 2);
       uint32_t bsw = bsw0 + sb * (SBB + 4);
       // FB super-blocks per flush: at most 3 FB additions into either accumulator
       for (; sb + FB - 1 < n_edge; sb += FB) {
 #pragma unroll
-        for (int u = 0; u < FB; u++) sb_edge<MB>(a0, a1, we + u * step, M, bsw + u * (SBB + 4));
-        flush2(hi, lo, a0, a1);
+        for (int u = 0; u < FB; u++) sb_edge<MB>(a, we + u * step, M, bsw + u * (SBB + 4));
+        flush2(hi, lo, a.x, a.y);
         we += FB * step, bsw += FB * (SBB + 4);
       }
       if (sb < n_edge) {
         for (; sb < n_edge; sb++) {
-          sb_edge<MB>(a0, a1, we, M, bsw);
+          sb_edge<MB>(a, we, M, bsw);
           we += step, bsw += SBB + 4;
         }
-        flush2(hi, lo, a0, a1);
+        flush2(hi, lo, a.x, a.y);
       }
     }
     for (; sb < n_all; sb++) {
-      sb_generic<MB>(a0, a1, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
+      sb_generic<MB>(a.x, a.y, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
                      bsw0 + sb * (SBB + 4), L, wr);
-      flush2(hi, lo, a0, a1);
+      flush2(hi, lo, a.x, a.y);
     }
   }
   __syncthreads();  // the next item and its copy flag are visible to every thread
@@ -894,7 +900,8 @@ __global__ void __launch_bounds__(32 * (NWS + kPcProducerWarps), NWS <= 14 ? 2 :
   bool live = false, plus_side = false, skip = false;
   uint32_t M = 0;
   WarpRange wr{0, 0, 0, 0};
-  float hi = 0.f, lo = 0.f, a0 = 0.f, a1 = 0.f;
+  float hi = 0.f, lo = 0.f;
+  float2 a = make_float2(0.f, 0.f);
   for (;;) {
     const int b = (int)(s & 1u);
     // one decision for the whole warp (a lane whose wait ran out fails every lane)
@@ -914,7 +921,7 @@ __global__ void __launch_bounds__(32 * (NWS + kPcProducerWarps), NWS <= 14 ? 2 :
       const HotItem it = items[cur];
       Wp = hdr + it.slot;
       skip = (h.flags & kPcSkip) != 0;
-      hi = lo = a0 = a1 = 0.f;
+      hi = lo = a.x = a.y = 0.f;
       if (!skip) {
         const WalkDev &W = *Wp;
         L = (int)W.L, N = (int)W.N;
@@ -945,49 +952,49 @@ __global__ void __launch_bounds__(32 * (NWS + kPcProducerWarps), NWS <= 14 ? 2 :
       const uint32_t bsw0 = tab_s0 + (uint32_t)b * (NSB * SBB);
       int sb = 0;
       {
-        const uint32_t *wu = win_f + (j + kt0), *wv = win_r + (j - kt0);
+        const uint32_t *wu = win_f + (j + kt0 - 2), *wv = win_r + (j - kt0 + 2);
         uint32_t bsw = bsw0;
         for (; sb + FB - 1 < n_int; sb += FB) {
 #pragma unroll
-          for (int u = 0; u < FB; u++) sb_interior<MB>(a0, a1, wu + u * kSbK, wv - u * kSbK, M, bsw + u * (SBB + 4));
-          flush2(hi, lo, a0, a1);
+          for (int u = 0; u < FB; u++) sb_interior<MB>(a, wu + u * kSbK, wv - u * kSbK, M, bsw + u * (SBB + 4));
+          flush2(hi, lo, a.x, a.y);
           wu += FB * kSbK, wv -= FB * kSbK, bsw += FB * (SBB + 4);
         }
         if (sb < n_int) {
           for (; sb < n_int; sb++) {
-            sb_interior<MB>(a0, a1, wu, wv, M, bsw);
+            sb_interior<MB>(a, wu, wv, M, bsw);
             wu += kSbK, wv -= kSbK, bsw += SBB + 4;
           }
-          flush2(hi, lo, a0, a1);
+          flush2(hi, lo, a.x, a.y);
         }
       }
       for (; sb < e0; sb++) {
-        sb_generic<MB>(a0, a1, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
+        sb_generic<MB>(a.x, a.y, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
                        bsw0 + sb * (SBB + 4), L, wr);
-        flush2(hi, lo, a0, a1);
+        flush2(hi, lo, a.x, a.y);
       }
       {
         const int step = plus_side ? kSbK : -kSbK;
-        const uint32_t *we = plus_side ? win_f + (j + kt0 + sb * kSbK) : win_r + (j - kt0 - sb * kSbK);
+        const uint32_t *we = plus_side ? win_f + (j + kt0 + sb * kSbK - 2) : win_r + (j - kt0 - sb * kSbK + 2);
         uint32_t bsw = bsw0 + sb * (SBB + 4);
         for (; sb + FB - 1 < n_edge; sb += FB) {
 #pragma unroll
-          for (int u = 0; u < FB; u++) sb_edge<MB>(a0, a1, we + u * step, M, bsw + u * (SBB + 4));
-          flush2(hi, lo, a0, a1);
+          for (int u = 0; u < FB; u++) sb_edge<MB>(a, we + u * step, M, bsw + u * (SBB + 4));
+          flush2(hi, lo, a.x, a.y);
           we += FB * step, bsw += FB * (SBB + 4);
         }
         if (sb < n_edge) {
           for (; sb < n_edge; sb++) {
-            sb_edge<MB>(a0, a1, we, M, bsw);
+            sb_edge<MB>(a, we, M, bsw);
             we += step, bsw += SBB + 4;
           }
-          flush2(hi, lo, a0, a1);
+          flush2(hi, lo, a.x, a.y);
         }
       }
       for (; sb < n_all; sb++) {
-        sb_generic<MB>(a0, a1, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
+        sb_generic<MB>(a.x, a.y, win_f, win_r, Ts, kt0, j, kt0 + sb * kSbK, kin, kout, plus_side, M,
                        bsw0 + sb * (SBB + 4), L, wr);
-        flush2(hi, lo, a0, a1);
+        flush2(hi, lo, a.x, a.y);
       }
     }
     __syncwarp();
