@@ -150,6 +150,7 @@ struct psl_ctx {
   int64_t next_id = 0;
   uint32_t hot_flush_sb = 8;  // super-blocks per block sum of the neighbourhood kernel
   bool tail_fused = false;    // every running walk is short: select..apply run as one kernel
+  bool hot_auto = false;      // the table kernel's block and tile follow the batch (neither was configured)
   bool lin = false;           // some running walk is long: scored by psl_lin.cu
   bool tables = false;        // some running walk is not
   bool alpha2 = false;        // every running walk has alpha1 = alpha2 = 2, L <= kA2MaxL: closed-form score
@@ -364,6 +365,7 @@ extern "C" int psl_init(const psl_config *cfg_in, psl_ctx **out) {
   if (cfg.arena && cfg.arena_bytes == 0) return fail(nullptr, PSL_EINVAL, "arena given without arena_bytes");
   psl_ctx *ctx = new psl_ctx();
   ctx->cfg = cfg;
+  ctx->hot_auto = cfg.hot_tile_sb == 0 && cfg.hot_threads == 0;
   if (ctx->cfg.hot_tile_sb == 0) ctx->cfg.hot_tile_sb = 32;
   if (ctx->cfg.hot_threads == 0) ctx->cfg.hot_threads = 256;
   auto bail = [&](int code) {
@@ -630,6 +632,28 @@ static int rebuild_active(psl_ctx *ctx) {
   }
   // Split every walk's k range into chunks when the neighbour blocks alone would leave
   // SMs idle (few walks, or a long walk on its own): aim for about four blocks per SM.
+  // Block and tile of the table kernel when the configuration leaves them open.  Blocks of 512 share each
+  // table between twice the neighbours, and a tile of 16 lets two of them fit an SM with the short
+  // walks' five tables a group, where one block of 256 with a tile of 32 is all that fits; a few walks
+  // fill more SMs with blocks of 256.  Microseconds a step, 256/32 against the choice here: 4096 walks of
+  // L = 1023 1692 / 718 (512/16), 64 of them 77.7 / 64.1, 256 of L = 4093 537 / 317, 2048 of L = 300
+  // 643 / 221; 64 of L = 8191 264 / 225 (512/32), 32 of them 160 / 164 and 64 of L = 300 49.0 / 52.2, so
+  // those keep 256/32.
+  if (ctx->hot_auto && !a2) {
+    uint64_t b512 = 0;
+    for (uint32_t s : ctx->active)
+      if (!ctx->h_hdr[s].lin && ctx->h_hdr[s].shard_count <= 1) b512 += (ctx->h_hdr[s].N + 511) / 512;
+    const bool big = fb == 4 ? 4 * b512 >= 3ull * ctx->sm_count : b512 >= 4ull * ctx->sm_count;
+    const int32_t t = big ? 512 : 256, sb = big && fb == 4 ? 16 : 32;
+    if (t != ctx->cfg.hot_threads || sb != ctx->cfg.hot_tile_sb) {
+      ctx->cfg.hot_threads = t;
+      ctx->cfg.hot_tile_sb = sb;
+      drop_graph(ctx);  // captured with another kernel variant
+    }
+  } else if (ctx->hot_auto && (ctx->cfg.hot_threads != 256 || ctx->cfg.hot_tile_sb != 32)) {
+    ctx->cfg.hot_threads = 256, ctx->cfg.hot_tile_sb = 32;
+    drop_graph(ctx);
+  }
   const uint32_t T_tab = (uint32_t)ctx->cfg.hot_threads * (a2 ? kA2PerThread : 1u);  // window positions per item
   std::vector<HotItem> quad;
   uint64_t nblocks = 0;
@@ -1336,6 +1360,7 @@ extern "C" int psl_autotune(psl_ctx *ctx, int reps) {
   if (rc) return rc;
   if (ctx->active_dirty && (rc = rebuild_active(ctx))) return rc;
   if (ctx->active.empty()) return fail(ctx, PSL_ESTATE, "no running walk to tune on");
+  ctx->hot_auto = false;
   if (!ctx->tables) return ctx->cfg.hot_threads | (ctx->cfg.hot_tile_sb << 16);  // one configuration
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
@@ -1387,6 +1412,7 @@ extern "C" int psl_hot_variant(psl_ctx *ctx, char *name, int32_t cap) {
 extern "C" int psl_set_hot_config(psl_ctx *ctx, int32_t threads, int32_t tile_sb) {
   if (!ctx || threads < 0 || tile_sb < 0 || !hot_config_supported((uint32_t)threads, (uint32_t)tile_sb))
     return PSL_EINVAL;
+  ctx->hot_auto = false;
   ctx->cfg.hot_threads = threads;
   ctx->cfg.hot_tile_sb = tile_sb;
   ctx->active_dirty = true;  // the block list depends on the block size
