@@ -10,9 +10,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libpsl.so")
-SOURCES = ["psl_kernels.cu", "psl_recheck.cu", "psl_tail.cu", "psl_hot.cu", "psl_lin.cu", "psl_alpha2.cu", "psl_runtime.cu",
+SOURCES = ["psl_kernels.cu", "psl_recheck.cu", "psl_tail.cu", "psl_tail_wide.cu", "psl_hot.cu", "psl_lin.cu", "psl_alpha2.cu", "psl_runtime.cu",
            "psl_static.cu", "psl_peak.cu"]
-HEADERS = [os.path.join(CSRC, "psl_internal.h"), os.path.join(CSRC, "psl_device.cuh"), os.path.join(CSRC, "psl_async.cuh"), os.path.join(CSRC, "psl_step.cuh"),
+HEADERS = [os.path.join(CSRC, "psl_internal.h"), os.path.join(CSRC, "psl_device.cuh"), os.path.join(CSRC, "psl_async.cuh"), os.path.join(CSRC, "psl_step.cuh"), os.path.join(CSRC, "psl_tail.cuh"),
            os.path.join(ROOT, "include", "psl.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2,-fvisibility=hidden",

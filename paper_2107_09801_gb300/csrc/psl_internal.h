@@ -135,6 +135,7 @@ struct LaunchCtx {
   uint32_t hot_flush_sb;   // super-blocks per block sum of the batched kernel (4 or 8)
   uint32_t sm_count;
   uint32_t alpha2;         // every running walk has alpha = 2 and L <= kA2MaxL: the closed-form score
+  uint32_t tail_wide;      // the fused step tail runs in wide blocks
   uint32_t lin;            // some walk is scored by psl_lin.cu
   uint32_t tables;         // some walk is scored by the tables of psl_hot.cu (or the closed form)
   uint32_t maxL;           // longest walk of an initialisation launch
@@ -167,6 +168,8 @@ cudaError_t launch_select(const LaunchCtx &c);
 cudaError_t launch_recheck(const LaunchCtx &c);
 cudaError_t launch_decide(const LaunchCtx &c);
 cudaError_t launch_step_tail(const LaunchCtx &c);  // select..apply in one kernel, short walks only
+cudaError_t launch_step_tail_wide(const LaunchCtx &c);  // psl_tail_wide.cu: the same in wider blocks
+cudaError_t prepare_tail_wide_kernel();
 constexpr uint32_t kA2MaxL = 4095;  // walks up to this length can take the alpha = 2 closed form
 constexpr uint32_t kA2PerThread = 4;  // window positions per thread of the closed-form kernel (per work item:
                                       // this many times the block size)
@@ -175,7 +178,7 @@ constexpr uint32_t kLinTilePos = 8192;   // window positions per k_lin tile
 // tile's chunks, about L + 20000 positions each (partners, and the rows that the tile's ends add).
 // 1024 walks with N = 6912, milliseconds a step, tables / psl_lin.cu: L = 16384 4.98 / 5.02, 18001 5.43 / 5.25,
 // 20001 5.94 / 5.44, 24577 7.18 / 5.94, 32767 9.29 / 6.81, 131071 38.3 / 21.2.
-inline bool lin_pays(uint32_t L, uint32_t N) {
+inline bool lin_pays(uint32_t L, uint32_t N) {  // L > 13488 whatever N
   const uint64_t tiles = (N + kLinTilePos - 1) / kLinTilePos;
   return (uint64_t)N * L >= 3300ull * ((uint64_t)L + 20000u) * tiles;
 }

@@ -150,6 +150,7 @@ struct psl_ctx {
   int64_t next_id = 0;
   uint32_t hot_flush_sb = 8;  // super-blocks per block sum of the neighbourhood kernel
   bool tail_fused = false;    // every running walk is short: select..apply run as one kernel
+  bool tail_wide = false;     // few walks: the fused tail runs in wide blocks
   bool hot_auto = false;      // the table kernel's block and tile follow the batch (neither was configured)
   bool lin = false;           // some running walk is long: scored by psl_lin.cu
   bool tables = false;        // some running walk is not
@@ -615,8 +616,13 @@ static int rebuild_active(psl_ctx *ctx) {
   for (uint32_t s : ctx->active)
     short_only = short_only && ctx->h_hdr[s].L <= kTailMaxL && ctx->h_hdr[s].N <= kTailMaxN &&
                  ctx->h_hdr[s].shard_count <= 1;
-  if (short_only != ctx->tail_fused) {
+  // One wave of eight-warp blocks (two fit an SM) is faster than one-warp blocks; more walks are not.
+  // Microseconds a step, one warp / eight: one walk of L = 1023 49.2 / 32.2, 304 of them 90.7 / 83.3, 608
+  // 139 / 145; 304 of L = 2047 157 / 139, of L = 300 53.5 / 52.8; one of L = 6000 (N = 2000) 127 / 40.
+  const bool wide = short_only && ctx->active.size() <= 2ull * ctx->sm_count;
+  if (short_only != ctx->tail_fused || wide != ctx->tail_wide) {
     ctx->tail_fused = short_only;
+    ctx->tail_wide = wide;
     drop_graph(ctx);  // captured with the other kernel sequence
   }
   // alpha = 2 batches of short walks take the closed-form score (unless the configuration
@@ -746,6 +752,7 @@ static LaunchCtx launch_ctx(psl_ctx *ctx, const uint32_t *d_list, Schedule *d_sc
   c.hot_flush_sb = ctx->hot_flush_sb;
   c.alpha2 = ctx->alpha2 ? 1u : 0u;
   c.lin = ctx->lin ? 1u : 0u;
+  c.tail_wide = ctx->tail_wide ? 1u : 0u;
   c.tables = ctx->tables ? 1u : 0u;
   c.sm_count = ctx->sm_count;
   c.stream = ctx->stream;

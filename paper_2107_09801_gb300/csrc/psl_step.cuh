@@ -148,7 +148,7 @@ __device__ __forceinline__ void apply_finish(WalkDev &W, uint32_t chunk, uint32_
     }
     W.psl = m;
     W.S_abs = s;
-    W.lin_sh = lin_shift(m, alpha, W.e);
+    if (L > (int)kTailMaxL) W.lin_sh = lin_shift(m, alpha, W.e);  // lin_pays() holds for no shorter walk
     W.alpha = alpha;
     if (need_F) {
       wide_store(W.F, Fs);
