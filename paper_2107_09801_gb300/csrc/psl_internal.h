@@ -149,6 +149,7 @@ cudaError_t prepare_hot_kernels();  // the neighbourhood kernels' part of it (ps
 cudaError_t prepare_recheck_kernel();  // psl_recheck.cu
 cudaError_t prepare_tail_kernel();     // psl_tail.cu
 cudaError_t launch_init_bits(const LaunchCtx &c);
+cudaError_t launch_pack_pm1(const LaunchCtx &c, const int8_t *seq);  // seq: ninit x maxL bytes on the device
 cudaError_t launch_autocorr(const LaunchCtx &c);
 cudaError_t launch_apply(const LaunchCtx &c);
 cudaError_t launch_hot_batched(const LaunchCtx &c);

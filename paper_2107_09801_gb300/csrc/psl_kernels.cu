@@ -52,6 +52,14 @@ __global__ void k_init_bits(WalkDev *hdr, const uint32_t *active) {
   if (idx == 0) W.psl = 0;
 }
 
+// Bits (1 for a negative value) of nseq +-1 sequences of L bytes, one warp a word.
+__global__ void __launch_bounds__(256) k_pack_pm1(const int8_t *__restrict__ seq, uint32_t L, uint32_t nw, WalkDev *hdr) {
+  const uint32_t i = blockIdx.x * 256u + threadIdx.x;
+  const bool neg = i < L && seq[(size_t)blockIdx.y * L + i] < 0;
+  const uint32_t word = __ballot_sync(0xffffffffu, neg);
+  if ((threadIdx.x & 31) == 0 && (i >> 5) < nw) hdr[blockIdx.y].bits[i >> 5] = word;
+}
+
 // C_k = (L-k) - 2 popc(x[0..L-k) xor x[k..L)) for one k per thread (Eq. 2 on packed bits);
 // PSL by atomicMax.  A block covers 256 consecutive k and streams the packed sequence
 // through shared memory in tiles of 2048 words: for thread k the partner window of word w
@@ -184,6 +192,11 @@ cudaError_t launch_init_bits(const LaunchCtx &c) {
   const uint32_t maxw = (c.maxL + 31) / 32 + 2 * kGuardWords;
   dim3 grid((maxw + 255) / 256, c.ninit);
   k_init_bits<<<grid, 256, 0, c.stream>>>(c.hdr, c.active);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pack_pm1(const LaunchCtx &c, const int8_t *seq) {
+  k_pack_pm1<<<dim3((c.maxL + 255) / 256, c.ninit), 256, 0, c.stream>>>(seq, c.maxL, (c.maxL + 31) / 32, c.hdr);
   return cudaGetLastError();
 }
 
