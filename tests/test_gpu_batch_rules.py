@@ -1,0 +1,32 @@
+"""Kernel variants chosen by the size of the batch give the same walks: blocks and tiles of the table
+kernel when the configuration leaves them open, and the width of the short walks' step tail."""
+import numpy as np
+import pytest
+
+import psl_workloads as W
+from helpers import have_gpu, same_decisions, submit_spec
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs a CUDA GPU")]
+
+
+def run(P, specs, keep, **kw):
+    with P.Context(arena_bytes=2 << 30, max_walks=len(specs), **kw) as ctx:
+        ids = [submit_spec(ctx, s) for s in specs]
+        name = ctx.hot_variant()
+        ctx.run()
+        return name, [(ctx.trace(ids[q], specs[q].budget), ctx.best(ids[q])) for q in keep]
+
+
+@pytest.mark.parametrize("L,walks,name", [(31, 400, "k_hot_batched<512,16,4>"), (1023, 400, "k_hot_batched<512,16,4>"),
+                                          (4095, 64, "k_hot_batched<512,16,4>"), (8191, 64, "k_hot_batched<512,32,8>")])
+def test_same_walks_in_any_batch(L, walks, name):
+    import paper_2107_09801_gb300 as P
+    specs = [W.WalkSpec(L=L, seed=q, alpha1=2 + q % 4, alpha2=8 + q % 5, budget=12, ls_lmt=2, topk=1 + q % 3) for q in range(walks)]
+    keep = [0, 1, walks // 2, walks - 1]
+    full, got = run(P, specs, keep, steps_per_graph=6)
+    assert full == name
+    few, want = run(P, [specs[q] for q in keep], range(len(keep)))  # 256 x 32, and eight-warp tail blocks
+    assert few.startswith("k_hot_batched<256,32")
+    for (tr, best), (tr0, best0) in zip(got, want):
+        assert same_decisions(tr, tr0)
+        assert best[0] == best0[0] and np.array_equal(best[1], best0[1])
