@@ -596,7 +596,9 @@ static int rebuild_active(psl_ctx *ctx) {
     WalkDev &h = ctx->h_hdr[s];
     const uint32_t was = h.lin;
     h.lin = use_lin && lin_pays(h.L, h.N) && h.shard_count <= 1 ? 1u : 0u;
-    if (h.lin && !was && h.moves > 0)  // the space of lin_y may hold partial scores of the tables
+    // the space of lin_y holds whatever the arena held, or partial scores of the tables (the autotuner runs them
+    // on walks that have not moved yet); from here on every score pass adds to zeros and leaves zeros
+    if (h.lin && !was)
       CK(cudaMemsetAsync(h.score_part + (size_t)kLinKsplitMax * h.N, 0, 8 * (size_t)h.N, ctx->stream));
     if (!h.lin) maxL = std::max(maxL, h.L);
     any_lin = any_lin || h.lin;

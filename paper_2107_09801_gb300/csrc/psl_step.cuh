@@ -120,11 +120,8 @@ __device__ __forceinline__ void apply_finish(WalkDev &W, uint32_t chunk, uint32_
   }
   if (keep_local)
     for (int w = threadIdx.x; w < nw; w += blockDim.x) W.bits_local[w] = W.bits[w];
-  if (mode == kModeInit) {
+  if (mode == kModeInit)
     for (int w = threadIdx.x; w < nw; w += blockDim.x) W.bits_best[w] = W.bits[w];
-    long long *Y = lin_y(W);  // every score pass adds to zeros and leaves zeros
-    for (int i = threadIdx.x; i < (int)W.N; i += blockDim.x) Y[i] = 0;
-  }
   if (threadIdx.x == 0) {
     int m = 0;
     float s = 0.f;

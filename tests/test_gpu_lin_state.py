@@ -1,0 +1,38 @@
+"""State that the correlation form (psl_lin.cu) shares with the tables: a walk's fixed-point sums lie in the
+space of the tables' last partial scores."""
+import numpy as np
+import pytest
+
+import psl_workloads as W
+from helpers import have_gpu, same_decisions, submit_spec
+import oracle as O
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not have_gpu(), reason="needs a CUDA GPU")]
+
+
+def wrapping_seed(L, n_lmt):
+    """A seed whose first window holds both ends of the sequence (their neighbours have the longest shifts)."""
+    return next(s for s in range(1000) if O.splitmix64(s, (L + 63) // 64) % L in range(L - n_lmt // 2 - 50, L - n_lmt // 2 + 50))
+
+
+@pytest.mark.parametrize("L", [30721, 46081])  # 16 k-chunks of 1920 and of 2880 shifts: the last two are full
+def test_walk_tuned_on_the_tables_before_its_first_move(L):
+    """The autotuner runs the tables, split 16 ways, on a walk that has made no move; with one tile for two SMs
+    the correlation then adds its shares to what lies in that space."""
+    import paper_2107_09801_gb300 as P
+    spec = W.WalkSpec(L=L, seed=wrapping_seed(L, 8192), alpha1=4, alpha2=13, budget=6, n_lmt=8192, ls_lmt=2)
+    res = []
+    for tune in (True, False):
+        with P.Context(arena_bytes=1 << 30, max_walks=1) as ctx:
+            wid = submit_spec(ctx, spec)
+            if tune:
+                ctx.autotune(reps=1)
+                assert ctx.hot_variant().startswith("k_hot")
+                ctx.set_max_sms(2)
+                assert ctx.hot_variant() == "k_lin + k_quad"
+            ctx.run()
+            assert ctx.poll(wid)["state"] == P.PSL_DONE
+            res.append((ctx.trace(wid, spec.budget), ctx.best(wid)))
+    (tr, best), (tr0, best0) = res
+    assert same_decisions(tr, tr0)
+    assert best[0] == best0[0] and np.array_equal(best[1], best0[1])
