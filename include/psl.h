@@ -330,6 +330,12 @@ PSL_API int psl_autocorr_static(const int8_t *seq_dev, uint32_t L, int32_t *C_de
  * flight.  PSL_ENOENT / PSL_EBUSY if the walk is unknown or not yet admitted. */
 PSL_API int psl_inject_stall(psl_ctx *ctx, int64_t id);
 
+/* The same for the other kind of wait: when the walk is scored by the correlation form, the
+ * kernel that multiplies on the tensor cores never announces the walk's products, so the
+ * threads that read them run out their (short) wait with products in flight.  A walk scored
+ * by the tables has no such wait and stalls as by psl_inject_stall. */
+PSL_API int psl_inject_product_stall(psl_ctx *ctx, int64_t id);
+
 /* Single-walk k-sharding over several ranks (one context per rank, typically one GPU each):
  * the parallel evaluation of Sec. 3 split over k, the sum of Eq. 4 being a sum over k.  A walk
  * submitted with shard_count = R > 1 (2 <= R <= min(16, ceil((L-1)/960)); the context must

@@ -73,7 +73,7 @@ class psl_alu_peak_t(ct.Structure):
 EXPORTED = ["psl_config_default", "psl_init", "psl_submit", "psl_submit_ex", "psl_step", "psl_poll", "psl_best",
             "psl_release", "psl_export_state", "psl_trace", "psl_autocorr", "psl_walk_bytes", "psl_shutdown",
             "psl_last_error", "psl_profile", "psl_profile_read", "psl_autotune", "psl_set_hot_config",
-            "psl_autocorr_static", "psl_inject_stall", "psl_set_max_sms",
+            "psl_autocorr_static", "psl_inject_stall", "psl_inject_product_stall", "psl_set_max_sms",
             "psl_best_fitness", "psl_transfer_bytes", "psl_set_steps_per_graph", "psl_alu_peak",
             "psl_shard_layout", "psl_shard_score", "psl_shard_select", "psl_shard_decide", "psl_best_many",
             "psl_hot_variant"]
@@ -116,6 +116,7 @@ def lib():
             "psl_hot_variant": (ct.c_int, [P, ct.c_char_p, ct.c_int32]),
             "psl_autocorr_static": (ct.c_int, [P, ct.c_uint32, P, P]),
             "psl_inject_stall": (ct.c_int, [P, ct.c_int64]),
+            "psl_inject_product_stall": (ct.c_int, [P, ct.c_int64]),
             "psl_set_max_sms": (ct.c_int, [P, ct.c_int32]),
             "psl_best_fitness": (ct.c_int, [P, ct.c_int64, P, P, P, ct.c_size_t]),
             "psl_transfer_bytes": (ct.c_int, [P, ct.POINTER(ct.c_uint64), ct.POINTER(ct.c_uint64)]),
@@ -441,9 +442,10 @@ class Context:
         return _check(self.h, lib().psl_shard_decide(self.h, wid, rc_words.ctypes.data if rc_words.size else None,
                                                       rc_words.size))
 
-    def inject_stall(self, wid: int) -> None:
-        """Test hook: the walk's next neighbourhood pass runs out its bounded waits."""
-        _check(self.h, lib().psl_inject_stall(self.h, wid))
+    def inject_stall(self, wid: int, products: bool = False) -> None:
+        """Test hook: the walk's next neighbourhood pass runs out its bounded waits on staged copies or,
+        with products, on the correlation form's tensor-core products."""
+        _check(self.h, (lib().psl_inject_product_stall if products else lib().psl_inject_stall)(self.h, wid))
 
     def profile(self, enable: bool | int = True) -> None:
         """True / 1: time every kernel; 2: the neighbourhood kernel only; False / 0: off."""

@@ -24,6 +24,7 @@ constexpr int kApplyPartStride = 32;  // u32 per apply-chunk partial record
 constexpr int kFlushBlockAdds = 64;   // FP32 additions per lane before a compensated flush
 constexpr int kKsplitMax = 16;        // most k-chunks one neighbour's score may be split into
 constexpr int kLinKsplitMax = 14;     // the same for walks scored by psl_lin.cu (the last two chunks' space holds lin_y)
+constexpr uint32_t kStallCopies = 1, kStallProducts = 2;  // WalkDev::inject_stall
 constexpr int kKchunkSbUnit = 32;     // k-chunks are whole multiples of 32 super-blocks (960 k)
 constexpr int kWinGuard = 32;         // entries before index 0 and past index L-1 of the partner windows
 
@@ -94,7 +95,7 @@ struct WalkDev {
   uint32_t ksplit, kchunk_sb;  // k-chunks of the neighbourhood kernel and their size (super-blocks)
   uint32_t kc_psl;             // the k-chunk whose blocks also compute the neighbours' exact PSL
   uint32_t lin;                // scored by psl_lin.cu (its own error bound)
-  uint32_t inject_stall;       // test hook: the next neighbourhood pass waits on copies never issued
+  uint32_t inject_stall;       // test hook: the next neighbourhood pass runs out a wait (kStallCopies, kStallProducts)
   float score_min, bound;
   uint32_t flips[kMaxFlips];
   uint32_t F[kWideLimbs], value_local[kWideLimbs], value_step[kWideLimbs];

@@ -33,7 +33,11 @@
 //     this rule differs from the exact boundary.
 // Roles: warps 0-7 expand S and drain the accumulators (256 TMEM columns per pipe), warps 8-13 build G
 // (a chunk each, a ring of stages per pipe), one thread of either of warps 14 and 15 issues a pipe's
-// products.  Every wait is bounded; a wait that runs out marks the walk failed and ends the block.
+// products.  Every wait on an mbarrier is bounded.  When one runs out, every role of the block leaves its
+// item, the walk whose item the epilogue was at gets its error, and the block starts again at its next item
+// with fresh barriers; if products may still be in flight, the walks of all its remaining items get theirs and
+// it ends.  k_quad then fails those walks: no status changes while k_lin runs, so that all threads of a block
+// agree on which items exist.
 //
 // What bounds it, at 304 walks of L = 131071 (N = 6912; two or three tiles per SM): k_lin 2.3 ms, the
 // tensor pipe active 57% of it (386 cycles a chunk; the rest is the issuing threads' instruction latency, the
@@ -112,9 +116,10 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+constexpr int kWaitLimit = 1 << 20;  // polls, each of which may itself suspend for a while
 // Bounded wait that also ends when another thread of the block gave up.
 __device__ __forceinline__ bool wait_or_err(uint32_t mbar, uint32_t parity, volatile int *err) {
-  for (int it = 0; it < (1 << 20); it++) {
+  for (int it = 0; it < kWaitLimit; it++) {
     if (mbar_try_wait(mbar, parity)) return true;
     if (*err) return false;
   }
@@ -123,11 +128,12 @@ __device__ __forceinline__ bool wait_or_err(uint32_t mbar, uint32_t parity, vola
 }
 // The same for a whole warp with one lane polling, `ns` apart; every lane then observes the completed
 // phase itself.
-__device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, volatile int *err, uint32_t ns) {
+__device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, volatile int *err, uint32_t ns,
+                                          int limit = kWaitLimit) {
   bool ok = true;
   if ((threadIdx.x & 31) == 0) {
     ok = false;
-    for (int it = 0; it < (1 << 20) && !*err; it++) {
+    for (int it = 0; it < limit && !*err; it++) {
       if ((ok = mbar_try_wait(mbar, parity))) break;
       __nanosleep(ns);
     }
@@ -145,13 +151,14 @@ __device__ __forceinline__ int floor_div64(int v) { return v >> 6; }
 struct LinTile {
   int L, jA, cnt, nb, rmin, rmax, qa, tau_lo, tau_hi, shares;
   int b_lo, b_hi, d_lo, d_hi;  // chunks with rows that take B: [b_lo, b_hi]; D: tau <= d_lo or tau >= d_hi
-  bool ok;
+  bool ok, stall;              // stall: the test hook withholds the item's products
 };
 
 __device__ __forceinline__ LinTile lin_tile(const WalkDev &W, const HotItem &it) {
   LinTile g;
   g.ok = false;
   if (W.status != kRunning) return g;
+  g.stall = (W.inject_stall & kStallProducts) != 0;
   const int L = (int)W.L, N = (int)W.N;
   const int f = ((int)W.start + 1) % L;
   int s0 = f, n0 = min(N, L - f), s1 = 0, n1 = N - n0;
@@ -274,70 +281,70 @@ __device__ __forceinline__ long long e_step(const float4 *__restrict__ T, int j,
   return d;
 }
 
-}  // namespace
+// What the roles of a block share.
+constexpr int kPipeBars = 2 * kStages + 2 * kSTiles + 2;  // full, empty, S full, S empty, accumulated, drained
+constexpr int kLinBars = kPipes * kPipeBars + 3;
+struct LinShared {
+  uint64_t bar[kLinBars];
+  long long seg[kLinEpiWarps], red[kLinEpiWarps];
+  uint32_t tmem;
+  uint32_t first, at;  // the block's first item, and the one the epilogue is at (past the last: their number)
+  int err, pending;    // a wait ran out; products may still be in flight
+  int limit;           // polls of the epilogue's wait for products
+};
+__shared__ LinShared s_lin;
 
-__global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotItem *items, const Schedule *sched) {
+__device__ __forceinline__ uint32_t lin_bars() { return (uint32_t)__cvta_generic_to_shared(s_lin.bar); }
+__device__ __forceinline__ uint32_t pipe_b(int pipe, uint32_t at) { return lin_bars() + 8u * ((uint32_t)(pipe * kPipeBars) + at); }
+__device__ __forceinline__ uint32_t full_b(int pipe, uint32_t s) { return pipe_b(pipe, s); }
+__device__ __forceinline__ uint32_t empty_b(int pipe, uint32_t s) { return pipe_b(pipe, kStages + s); }
+__device__ __forceinline__ uint32_t sfull_b(int pipe, uint32_t s) { return pipe_b(pipe, 2 * kStages + s); }
+__device__ __forceinline__ uint32_t sempty_b(int pipe, uint32_t s) { return pipe_b(pipe, 2 * kStages + kSTiles + s); }
+__device__ __forceinline__ uint32_t accf_b(int pipe) { return pipe_b(pipe, 2 * kStages + 2 * kSTiles); }
+__device__ __forceinline__ uint32_t drain_b(int pipe) { return pipe_b(pipe, 2 * kStages + 2 * kSTiles + 1); }
+__device__ __forceinline__ uint32_t win_b(uint32_t s) { return lin_bars() + 8u * (kPipes * kPipeBars + s); }
+__device__ __forceinline__ uint32_t acce_b() { return lin_bars() + 8u * (kPipes * kPipeBars + 2); }
+
+__device__ __forceinline__ void lin_init_bars() {
+  for (int pipe = 0; pipe < kPipes; pipe++) {
+    for (uint32_t s = 0; s < kStages; s++) {
+      mbar_init(full_b(pipe, s), 32);
+      mbar_init(empty_b(pipe, s), 1);
+    }
+    for (uint32_t s = 0; s < kSTiles; s++) {
+      mbar_init(sfull_b(pipe, s), 32 * kLinEpiWarps);
+      mbar_init(sempty_b(pipe, s), 1);
+    }
+    mbar_init(accf_b(pipe), 1);
+    mbar_init(drain_b(pipe), 1);
+    mbar_init(win_b((uint32_t)pipe), 32 * kLinEpiWarps);
+  }
+  mbar_init(acce_b(), 32 * kLinEpiWarps);
+  fence_mbar_init();
+  s_lin.err = s_lin.pending = 0;
+}
+
+// The block's items from s_lin.first on (every gridDim.x-th), until they are done or a wait runs out.
+// A call of its own: inlined into the loop of k_lin, the epilogue spills (304 walks of L = 131071: 5.96 ms a
+// step, 5.87 so).
+__device__ __noinline__ void lin_items(WalkDev *hdr, const HotItem *items, uint32_t nitems) {
   extern __shared__ __align__(128) uint8_t lin_smem[];
-  constexpr int kPipeBars = 2 * kStages + 2 * kSTiles + 2;  // full, empty, S full, S empty, accumulated, drained
-  __shared__ __align__(8) uint64_t s_bar[kPipes * kPipeBars + 3];
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_err;
-  __shared__ long long s_seg[kLinEpiWarps];
-  __shared__ long long s_red[kLinEpiWarps];
+  LinShared &s = s_lin;
   const uint32_t base = ((uint32_t)__cvta_generic_to_shared(lin_smem) + 127u) & ~127u;
   const uint32_t win_s = base, stile_s = win_s + 2 * kWinBytes, h_s = stile_s + kPipes * kSTiles * kSTileBytes;
-  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(s_bar);
-  auto pipe_b = [&](int pipe, uint32_t at) { return bar + 8u * ((uint32_t)(pipe * kPipeBars) + at); };
-  auto full_b = [&](int pipe, uint32_t s) { return pipe_b(pipe, s); };
-  auto empty_b = [&](int pipe, uint32_t s) { return pipe_b(pipe, kStages + s); };
-  auto sfull_b = [&](int pipe, uint32_t s) { return pipe_b(pipe, 2 * kStages + s); };
-  auto sempty_b = [&](int pipe, uint32_t s) { return pipe_b(pipe, 2 * kStages + kSTiles + s); };
-  auto accf_b = [&](int pipe) { return pipe_b(pipe, 2 * kStages + 2 * kSTiles); };
-  auto drain_b = [&](int pipe) { return pipe_b(pipe, 2 * kStages + 2 * kSTiles + 1); };
-  auto win_b = [&](uint32_t s) { return bar + 8u * (kPipes * kPipeBars + s); };
-  const uint32_t acce_b = bar + 8u * (kPipes * kPipeBars + 2);
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) {
-    for (int pipe = 0; pipe < kPipes; pipe++) {
-      for (uint32_t s = 0; s < kStages; s++) {
-        mbar_init(full_b(pipe, s), 32);
-        mbar_init(empty_b(pipe, s), 1);
-      }
-      for (uint32_t s = 0; s < kSTiles; s++) {
-        mbar_init(sfull_b(pipe, s), 32 * kLinEpiWarps);
-        mbar_init(sempty_b(pipe, s), 1);
-      }
-      mbar_init(accf_b(pipe), 1);
-      mbar_init(drain_b(pipe), 1);
-      mbar_init(win_b((uint32_t)pipe), 32 * kLinEpiWarps);
-    }
-    mbar_init(acce_b, 32 * kLinEpiWarps);
-    fence_mbar_init();
-    s_err = 0;
-  }
-  if (warp == kLinEpiWarps + kLinBuilders) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(&s_tmem))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = s_tmem;
-  const uint32_t nitems = sched->nlin;
-  const HotItem *lin_items = items + sched->nitems + sched->nquad;
-  volatile int *err = &s_err;
-
+  const uint32_t tmem = s.tmem;
+  volatile int *err = &s.err;
   if (warp < kLinEpiWarps) {
     // ---------------- expand S, drain the accumulators, write Y ----------------
     uint32_t sg = 0, sq[kPipes] = {0, 0};  // segments, and chunks with S tiles of either pipe, so far
     bool ok = true;
-    for (uint32_t n = blockIdx.x; ok && n < nitems; n += gridDim.x) {
-      const HotItem it = lin_items[n];
-      WalkDev &W = hdr[it.slot];
+    for (uint32_t n = s.first; ok && n < nitems; n += gridDim.x) {
+      const HotItem it = items[n];
+      const WalkDev &W = hdr[it.slot];
       const LinTile g = lin_tile(W, it);
       if (!g.ok) continue;
+      if (tid == 0) s.at = n, s.limit = g.stall ? 64 : kWaitLimit;
       const int L = g.L;
       const uint32_t *__restrict__ bits = W.bits;
       const float4 *__restrict__ T = W.T;
@@ -434,10 +441,10 @@ __global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotI
             es += __shfl_xor_sync(0xffffffffu, es, o);
             e += __shfl_xor_sync(0xffffffffu, e, o);
           }
-          if (lane == 0) s_red[warp] = es, s_seg[warp] = e;
+          if (lane == 0) s.red[warp] = es, s.seg[warp] = e;
           named_sync<1, 32 * kLinEpiWarps>();
           long long run = 0;
-          for (int w = 0; w < kLinEpiWarps; w++) run += s_red[w] + (w < warp ? s_seg[w] : 0);
+          for (int w = 0; w < kLinEpiWarps; w++) run += s.red[w] + (w < warp ? s.seg[w] : 0);
 #pragma unroll 4
           for (int x = w0 + lane; x - lane < min(w0 + kTilePos / kLinEpiWarps, g.cnt); x += 32) {
             long long v = first && x > 0 && x < g.cnt ? e_step(T, g.jA + x, L, s2) : 0;
@@ -452,7 +459,8 @@ __global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotI
           }
           __threadfence_block();  // the sums are read back by other threads of the block, after the barrier below
         }
-        for (int pipe = 0; pipe < kPipes; pipe++) ok = ok && warp_wait(accf_b(pipe), sg & 1u, err, 100);
+        for (int pipe = 0; pipe < kPipes; pipe++)
+          ok = ok && warp_wait(accf_b(pipe), sg & 1u, err, 100, *(volatile int *)&s.limit);
         ok = !named_any(1, 32 * kLinEpiWarps, !ok);  // one decision for all eight warps
         if (!ok) break;
         tc_fence_after();
@@ -478,30 +486,25 @@ __global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotI
           }
         }
         tc_fence_before();
-        mbar_arrive(acce_b);
+        mbar_arrive(acce_b());
       }
-      if (!ok) {
-        if (tid == 0) {
-          W.error = (uint32_t)-5;  // PSL_ETIMEOUT of the library header
-          W.status = kError;
-        }
-        break;
-      }
+      if (!ok) break;
 #pragma unroll
       for (int q = 0; q < 32; q++) {
         // column 32 half + q' holds a = 63 - (32 half + q'): ascending positions are descending columns
         const int x = x0 + q, j = g.jA + x, i = win_index(j);
         if (x < g.cnt) add_y(i, getbit(bits, j) ? -acc[31 - q] : acc[31 - q], true);
       }
-      named_sync<1, 32 * kLinEpiWarps>();  // s_seg and s_red are free for the next item
+      named_sync<1, 32 * kLinEpiWarps>();  // s.seg and s.red are free for the next item
     }
+    if (ok && tid == 0) s.at = nitems;
   } else if (warp < kLinEpiWarps + kLinBuilders) {
     // ---------------- build G: a chunk per warp ----------------
     const int pipe = (warp - kLinEpiWarps) / kPipeBuilders, bw = (warp - kLinEpiWarps) % kPipeBuilders;
     uint32_t q0 = 0, c0 = 0;  // the pipe's products, and its chunks modulo its builders, of the items before
     bool ok = true;
-    for (uint32_t n = blockIdx.x; ok && n < nitems; n += gridDim.x) {
-      const HotItem it = lin_items[n];
+    for (uint32_t n = s.first; ok && n < nitems; n += gridDim.x) {
+      const HotItem it = items[n];
       const WalkDev &W = hdr[it.slot];
       const LinTile g = lin_tile(W, it);
       if (!g.ok) continue;
@@ -586,14 +589,15 @@ __global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotI
     const uint32_t d = tmem + (uint32_t)pipe * kAccCols, hp_s = h_s + (uint32_t)(pipe * kStages) * kHBytes,
                    sp_s = stile_s + (uint32_t)(pipe * kSTiles) * kSTileBytes;
     uint32_t st = 0, ph = 0, ss = 0, sph = 0, sg = 0;  // stage and S tile with their phases, segment
+    uint32_t nacc = 0;                                 // segments announced
     bool ok = true, ready = false;                     // the stage is full
-    for (uint32_t n = blockIdx.x; ok && n < nitems; n += gridDim.x) {
-      const HotItem it = lin_items[n];
+    for (uint32_t n = s.first; ok && n < nitems; n += gridDim.x) {
+      const HotItem it = items[n];
       const LinTile g = lin_tile(hdr[it.slot], it);
       if (!g.ok) continue;
       for (int t0 = g.tau_lo; ok && t0 <= g.tau_hi; t0 += kSegTau, sg++) {
         const uint32_t buf = sg & 1u;
-        if (sg >= 1) ok = wait_or_err(acce_b, (sg - 1u) & 1u, err);
+        if (sg >= 1) ok = wait_or_err(acce_b(), (sg - 1u) & 1u, err);
         if (ok) ok = wait_or_err(win_b(buf), (sg >> 1) & 1u, err);
         if (!ok) break;
         bool acc = false;
@@ -624,19 +628,60 @@ __global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotI
             }
           }
         }
-        if (ok) mma_commit(accf_b(pipe));
+        if (ok && !g.stall) mma_commit(accf_b(pipe)), nacc++;
       }
     }
-    // nothing is in flight when the accumulators are given back
+    // nothing is in flight when the accumulators are given back or the barriers set up again: no product, and no
+    // arrival of a commit (the last one on each barrier; a parity that no commit has reached yet reads complete)
     mma_commit(drain_b(pipe));
-    mbar_wait_bounded(drain_b(pipe), 0);
+    bool done = mbar_wait_bounded(drain_b(pipe), 0) && mbar_wait_bounded(accf_b(pipe), (nacc - 1u) & 1u);
+    for (uint32_t q = 0; q < kStages; q++) done = done && mbar_wait_bounded(empty_b(pipe, q), q < st ? ph : ph ^ 1u);
+    for (uint32_t q = 0; q < kSTiles; q++) done = done && mbar_wait_bounded(sempty_b(pipe, q), q < ss ? sph : sph ^ 1u);
+    if (!done) s.pending = s.err = 1;
   }
   __syncwarp();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == kLinEpiWarps + kLinBuilders)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kLinThreads, 1) k_lin(WalkDev *hdr, const HotItem *all_items, const Schedule *sched) {
+  if (threadIdx.x == 0) {
+    lin_init_bars();
+    s_lin.first = blockIdx.x;
+  }
+  const bool alloc = threadIdx.x / 32 == kLinEpiWarps + kLinBuilders;
+  if (alloc) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(&s_lin.tmem))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const HotItem *items = all_items + sched->nitems + sched->nquad;
+  const uint32_t nitems = sched->nlin;
+  for (;;) {  // (a second time only after a wait ran out)
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    lin_items(hdr, items, nitems);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (!s_lin.err) break;
+    const uint32_t at = s_lin.at;
+    const bool pending = s_lin.pending != 0;
+    if (threadIdx.x == 0)
+      for (uint32_t n = at; n < nitems && (pending || n == at); n += gridDim.x)
+        hdr[items[n].slot].error = (uint32_t)-5;  // PSL_ETIMEOUT of the library header
+    __syncthreads();  // every thread has read the flags
+    if (pending) break;
+    if (threadIdx.x == 0) {
+      for (uint32_t b = 0; b < kLinBars; b++) mbar_inval(lin_bars() + 8u * b);
+      lin_init_bars();
+      s_lin.first = at + gridDim.x;
+    }
+  }
+  if (alloc)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(s_lin.tmem) : "memory");
 }
 
 // ------------------------------------------------------------------------------------
@@ -787,7 +832,8 @@ __global__ void __launch_bounds__(kQThreads, 2) k_quad(WalkDev *hdr, const HotIt
         s_item = nx;
         s_prun = 0, s_pstall = 0;
         if (nx < nquad) {
-          const WalkDev &Wn = hdr[items[nx].slot];
+          WalkDev &Wn = hdr[items[nx].slot];
+          if (Wn.error) Wn.status = kError;  // k_lin ran out a wait over the walk
           s_prun = Wn.status == kRunning ? 1 : 0;
           s_pstall = Wn.inject_stall ? 1 : 0;
         }

@@ -1443,16 +1443,18 @@ extern "C" int psl_set_max_sms(psl_ctx *ctx, int32_t max_sms) {
   return (int)n;
 }
 
-extern "C" int psl_inject_stall(psl_ctx *ctx, int64_t id) {
+static int inject(psl_ctx *ctx, int64_t id, uint32_t kind) {
   if (!ctx) return PSL_EINVAL;
   HostWalk *w = find(ctx, id);
   if (!w) return PSL_ENOENT;
   if (w->slot < 0) return PSL_EBUSY;
-  const uint32_t one = 1;
-  CK(xfer(ctx, (char *)(ctx->d_hdr + w->slot) + offsetof(WalkDev, inject_stall), &one, 4, cudaMemcpyHostToDevice));
+  CK(xfer(ctx, (char *)(ctx->d_hdr + w->slot) + offsetof(WalkDev, inject_stall), &kind, 4, cudaMemcpyHostToDevice));
   CK(cudaStreamSynchronize(ctx->stream));
   return PSL_OK;
 }
+
+extern "C" int psl_inject_stall(psl_ctx *ctx, int64_t id) { return inject(ctx, id, kStallCopies); }
+extern "C" int psl_inject_product_stall(psl_ctx *ctx, int64_t id) { return inject(ctx, id, kStallProducts); }
 
 // ---------------------------------------------------------------------------------
 // single-walk k-sharding: one step split into the rank's share of the work and two
