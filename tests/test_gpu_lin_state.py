@@ -69,3 +69,17 @@ def test_a_wait_that_runs_out_fails_only_that_walk(products, stall):
         else:
             assert st["state"] == P.PSL_DONE
             assert same_decisions(tr, tr0) and best[0] == best0[0] and np.array_equal(best[1], best0[1])
+
+
+@pytest.mark.parametrize("L,n_lmt,sms", [(30721, 8192, 2), (65537, 4500, 2), (70001, 6912, 2), (90001, 8193, 4),
+                                         (33000, 12001, 4), (40000, 40000, 10)])
+def test_partners_split_over_two_items(L, n_lmt, sms):
+    """Half as many tiles as SMs: two items share a tile's partners and add their sums up."""
+    import paper_2107_09801_gb300 as P
+    spec = W.WalkSpec(L=L, seed=wrapping_seed(L, n_lmt) if n_lmt < L else 5, alpha1=4, alpha2=13, budget=6, n_lmt=n_lmt,
+                      ls_lmt=2)
+    name, ((st, tr, best),) = run_stalled(P, [spec], [], False, max_sms=sms)
+    assert name == "k_lin + k_quad" and st["state"] == P.PSL_DONE
+    _, ((_, tr0, best0),) = run_stalled(P, [spec], [], False)
+    assert same_decisions(tr, tr0)
+    assert best[0] == best0[0] and np.array_equal(best[1], best0[1])
