@@ -176,10 +176,11 @@ constexpr uint32_t kA2MaxL = 4095;  // walks up to this length can take the alph
 constexpr uint32_t kA2PerThread = 4;  // window positions per thread of the closed-form kernel (per work item:
                                       // this many times the block size)
 constexpr uint32_t kLinTilePos = 8192;   // window positions per k_lin tile
-// Walks that psl_lin.cu scores faster than the tables: it saves lookups in proportion to N L and costs a
-// tile's chunks, about L + 20000 positions each (partners, and the rows that the tile's ends add).
-// 1024 walks with N = 6912, milliseconds a step, tables / psl_lin.cu: L = 16384 4.98 / 5.02, 18001 5.43 / 5.25,
-// 20001 5.94 / 5.44, 24577 7.18 / 5.94, 32767 9.29 / 6.81, 131071 38.3 / 21.2.
+// Walks that psl_lin.cu scores faster than the tables in a large batch: it saves lookups in proportion to N L
+// and costs a tile's chunks, about L + 20000 positions each (partners, and the rows that the tile's ends add).
+// 1024 walks with N = 6912, milliseconds a step, tables / psl_lin.cu: L = 16384 4.91 / 4.97, 20001 5.86 / 5.37,
+// 24577 7.07 / 5.84, 32767 9.15 / 6.74, 131071 35.2 / 18.0.  (Whether a batch fills the SMs evenly enough is
+// lin_worth in psl_runtime.cu.)
 inline bool lin_pays(uint32_t L, uint32_t N) {  // L > 13488 whatever N
   const uint64_t tiles = (N + kLinTilePos - 1) / kLinTilePos;
   return (uint64_t)N * L >= 3300ull * ((uint64_t)L + 20000u) * tiles;

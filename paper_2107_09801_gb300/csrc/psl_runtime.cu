@@ -572,6 +572,58 @@ static void fill_header(psl_ctx *ctx, HostWalk &w, WalkDev &h) {
   h.rng_ctr = (p.L + 63) / 64;
 }
 
+// k_lin's tiles of a walk: one more where the window may wrap around the end
+static uint32_t lin_tiles(uint32_t L, uint32_t N) { return (N + kLinTilePos - 1) / kLinTilePos + (N < L ? 1u : 0u); }
+
+// Whether psl_lin.cu beats the tables on the walks `cand` (slots, in the order of k_lin's items) by enough.
+// k_lin's blocks take whole items in turn, so what counts is the block with the most: the last wave of items,
+// and where the windows that wrap around the end put their second tile.  That block is found here from the
+// assignment itself, for a few fixed draws of the window starts; a tile of c positions is (L + 3 c) / 64 chunks
+// (the partners, the rows added by its ends, and the chunks done twice, which fall to one of the tile's shares).
+// The constants are fitted to the steps of both forms in 379 batches of 38 to 1024 walks, L = 13500 to 131071,
+// N = 3600 to 16384, on 152 SMs: lookups saved 0.029 us for 10^6 of N L less 0.2 us for 1000 of N, 0.28 us a
+// chunk, 60 us for the launch.  In 18 of them the rule takes the slower form, by 2% to 16% (it misses gains just
+// past a full wave and for the smallest N); lin_pays and half the SMs alone take it in 77, by up to 57%.
+// Milliseconds a step of N = 6912, tables / psl_lin.cu: L = 20001: 80 walks 0.56 / 0.72, 151 0.93 / 0.98, 152
+// 0.93 / 0.85, 160 1.00 / 1.17, 304 1.80 / 1.61, 320 1.90 / 1.95; L = 32767: 76 0.74 / 0.68, 90 0.90 / 0.98, 160
+// 1.54 / 1.47; L = 65535: 90 1.70 / 1.50.
+static bool lin_worth(const psl_ctx *ctx, const std::vector<uint32_t> &cand, uint32_t split) {
+  const uint32_t sms = ctx->sm_count;
+  double saved = 0.0;
+  for (uint32_t s : cand) saved += ctx->h_hdr[s].N * (2.9e-8 * ctx->h_hdr[s].L - 2.0e-4);
+  constexpr int kDraws = 4;
+  double longest = 0.0;
+  uint64_t x = 1;
+  std::vector<double> load(sms);
+  std::vector<uint32_t> first(cand.size());  // positions of the window before the end of the sequence
+  for (int d = 0; d < kDraws; d++) {
+    std::fill(load.begin(), load.end(), 0.0);
+    for (size_t w = 0; w < cand.size(); w++) {
+      const WalkDev &h = ctx->h_hdr[cand[w]];
+      x = x * 6364136223846793005ull + 1442695040888963407ull;
+      first[w] = h.N == h.L ? h.N : std::min<uint32_t>(h.N, h.L - (uint32_t)((x >> 33) % h.L));
+    }
+    size_t n = 0;
+    bool more = true;
+    for (uint32_t t = 0; more; t++) {
+      more = false;
+      for (size_t w = 0; w < cand.size(); w++) {
+        const WalkDev &h = ctx->h_hdr[cand[w]];
+        const uint32_t nt = lin_tiles(h.L, h.N), t0 = (first[w] + kLinTilePos - 1) / kLinTilePos;
+        more = more || t + 1 < nt;
+        if (t >= nt) continue;
+        const int64_t left = t < t0 ? (int64_t)first[w] - (int64_t)t * kLinTilePos
+                                    : (int64_t)(h.N - first[w]) - (int64_t)(t - t0) * kLinTilePos;
+        const double c = (double)std::min<int64_t>(left, kLinTilePos);
+        for (uint32_t q = 0; q < split; q++, n++)
+          if (c > 0) load[n % sms] += ((double)h.L + c) / split + 2.0 * c;
+      }
+    }
+    longest += *std::max_element(load.begin(), load.end()) / kDraws;
+  }
+  return saved * 152.0 / sms >= 1.03 * (60.0 + 0.28 / 64.0 * longest);
+}
+
 static int rebuild_active(psl_ctx *ctx) {
   ctx->active.clear();
   for (auto &kv : ctx->walks)
@@ -584,18 +636,26 @@ static int rebuild_active(psl_ctx *ctx) {
   ctx->max_chunk_rc = 1;
   // short walks run their few super-blocks with shorter block sums (less unrolled code)
   uint32_t maxL = 0;
-  // Long walks are scored by psl_lin.cu when their tiles fill at least half the SMs, all others by the
-  // tables of psl_hot.cu.  Milliseconds a step, tables / psl_lin.cu: 76 walks of L = 131071 2.75 / 1.84, of
-  // L = 32767 0.76 / 0.69; one walk of L = 131071 (split over the SMs) 0.13 / 0.20.
+  // Long walks are scored by psl_lin.cu when their tiles fill at least half the SMs and fill them evenly enough,
+  // all others by the tables of psl_hot.cu.  (One walk of L = 131071 takes 0.13 ms a step by the tables and 0.20
+  // split over the SMs; 38 walks of L = 65535 0.85 and 0.65, of L = 20001 0.32 and 0.36.)
+  std::vector<uint32_t> cand;
   uint64_t tiles = 0;
-  for (uint32_t s : ctx->active)
-    if (lin_pays(ctx->h_hdr[s].L, ctx->h_hdr[s].N)) tiles += (ctx->h_hdr[s].N + kLinTilePos - 1) / kLinTilePos;
-  const bool use_lin = ctx->cfg.form == PSL_FORM_BATCHED && 2 * tiles >= ctx->sm_count;
+  if (ctx->cfg.form == PSL_FORM_BATCHED)
+    for (uint32_t s : ctx->active) {
+      const WalkDev &h = ctx->h_hdr[s];
+      if (!lin_pays(h.L, h.N) || h.shard_count > 1) continue;
+      cand.push_back(s);
+      tiles += (h.N + kLinTilePos - 1) / kLinTilePos;
+    }
+  // two items share a tile's partners when that fills the SMs
+  const uint32_t lin_split = tiles ? (uint32_t)std::max<uint64_t>(1, ctx->sm_count / tiles) : 1u;
+  const bool use_lin = tiles && 2 * tiles >= ctx->sm_count && lin_worth(ctx, cand, lin_split);
   bool any_lin = false, any_tab = false;
   for (uint32_t s : ctx->active) {
     WalkDev &h = ctx->h_hdr[s];
     const uint32_t was = h.lin;
-    h.lin = use_lin && lin_pays(h.L, h.N) && h.shard_count <= 1 ? 1u : 0u;
+    h.lin = use_lin && h.shard_count <= 1 && lin_pays(h.L, h.N) ? 1u : 0u;
     // the space of lin_y holds whatever the arena held, or partial scores of the tables (the autotuner runs them
     // on walks that have not moved yet); from here on every score pass adds to zeros and leaves zeros
     if (h.lin && !was)
@@ -694,12 +754,10 @@ static int rebuild_active(psl_ctx *ctx) {
     ctx->max_chunk_apply = std::max(ctx->max_chunk_apply, h.nchunk_apply);
     ctx->max_chunk_rc = std::max(ctx->max_chunk_rc, h.nchunk_rc);
   }
-  // k_lin's items: the tiles of every walk (one more where the window may wrap around the end), each
-  // walk's partners split over several items when the tiles alone would leave SMs idle
+  // k_lin's items: the tiles of every walk (one more where the window may wrap around the end)
   const size_t nitems = items.size(), nquad = quad.size();
   items.insert(items.end(), quad.begin(), quad.end());
   if (any_lin) {
-    const uint32_t split = (uint32_t)std::max<uint64_t>(1, ctx->sm_count / tiles);
     // tile 0 of every walk first: most windows end there, and the blocks take the items in turn
     bool more = true;
     for (uint32_t t = 0; more; t++) {
@@ -707,9 +765,9 @@ static int rebuild_active(psl_ctx *ctx) {
       for (uint32_t s : ctx->active) {
         const WalkDev &h = ctx->h_hdr[s];
         if (!h.lin) continue;
-        const uint32_t nt = (h.N + kLinTilePos - 1) / kLinTilePos + (h.N < h.L ? 1u : 0u);
+        const uint32_t nt = lin_tiles(h.L, h.N);
         more = more || t + 1 < nt;
-        for (uint32_t c = 0; t < nt && c < split; c++) items.push_back(HotItem{s, t, c, split});
+        for (uint32_t c = 0; t < nt && c < lin_split; c++) items.push_back(HotItem{s, t, c, lin_split});
       }
     }
   }

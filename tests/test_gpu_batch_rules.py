@@ -30,3 +30,18 @@ def test_same_walks_in_any_batch(L, walks, name):
     for (tr, best), (tr0, best0) in zip(got, want):
         assert same_decisions(tr, tr0)
         assert best[0] == best0[0] and np.array_equal(best[1], best0[1])
+
+
+@pytest.mark.parametrize("L,walks,lin", [(13500, 100, False), (20001, 80, False), (20001, 152, True), (20001, 160, False),
+                                         (20001, 304, True), (32767, 90, False), (32767, 152, True), (65535, 77, True)])
+def test_correlation_form_where_its_tiles_fill_the_sms(L, walks, lin):
+    """On 152 SMs: a last wave of few tiles costs more than the lookups it saves."""
+    import torch
+    import paper_2107_09801_gb300 as P
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the line depends on the number of SMs")
+    n_lmt = 8192 if L == 13500 else 6912
+    with P.Context(arena_bytes=walks * P.psl_walk_bytes(L, n_lmt, 0) + (64 << 20), max_walks=walks) as ctx:
+        for q in range(walks):
+            ctx.submit_ex(L, q, 4, 13, 10, n_lmt=n_lmt)
+        assert (ctx.hot_variant() == "k_lin + k_quad") == lin
