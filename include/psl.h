@@ -271,7 +271,9 @@ PSL_API int psl_alu_peak(int32_t device, void *stream, psl_alu_peak_t *out);
  * tables into one of two buffers while the other warps score) on the walks now
  * running, reps launches each, and keeps the fastest for this context.  The timed
  * launches only recompute window scores that the next step recomputes, so no result
- * changes.  Returns threads | (tile_sb << 16) of the choice, PSL_ESTATE when no walk
+ * changes.  Walks scored by the correlation form have one configuration: when all of them
+ * are, nothing is timed or kept and the present setting is returned.  Returns
+ * threads | (tile_sb << 16) of the choice, PSL_ESTATE when no walk
  * is running, PSL_EINVAL for the plain form or reps < 1. */
 PSL_API int psl_autotune(psl_ctx *ctx, int reps);
 

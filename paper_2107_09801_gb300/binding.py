@@ -366,7 +366,8 @@ class Context:
 
     def autotune(self, reps: int = 3, cache: str | None = None) -> tuple[int, int]:
         """Picks the neighbourhood-kernel configuration for the running walks.  With a
-        cache file, a previous choice for the same GPU and length bucket is reused."""
+        cache file, a previous choice for the same GPU and length bucket is reused.  (Walks that
+        the correlation form scores leave nothing to choose, and nothing to store.)"""
         key = None
         if cache:
             import json
@@ -381,7 +382,7 @@ class Context:
                 self._set_hot(t, sb)
                 return t, sb
         t, sb = psl_autotune(self.h, reps)
-        if cache:
+        if cache and self.hot_variant() != "k_lin + k_quad":
             table[key] = [t, sb]
             tmp = cache + ".tmp"
             with open(tmp, "w") as f:

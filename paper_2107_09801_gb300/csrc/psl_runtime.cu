@@ -1430,8 +1430,8 @@ extern "C" int psl_autotune(psl_ctx *ctx, int reps) {
   if (rc) return rc;
   if (ctx->active_dirty && (rc = rebuild_active(ctx))) return rc;
   if (ctx->active.empty()) return fail(ctx, PSL_ESTATE, "no running walk to tune on");
+  if (!ctx->tables) return ctx->cfg.hot_threads | (ctx->cfg.hot_tile_sb << 16);  // psl_lin.cu: nothing to choose
   ctx->hot_auto = false;
-  if (!ctx->tables) return ctx->cfg.hot_threads | (ctx->cfg.hot_tile_sb << 16);  // one configuration
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
   CK(cudaEventCreate(&b));

@@ -45,3 +45,20 @@ def test_correlation_form_where_its_tiles_fill_the_sms(L, walks, lin):
         for q in range(walks):
             ctx.submit_ex(L, q, 4, 13, 10, n_lmt=n_lmt)
         assert (ctx.hot_variant() == "k_lin + k_quad") == lin
+
+
+def test_autotuner_leaves_the_choice_open_when_there_is_none(tmp_path):
+    """Tuning a batch that the correlation form scores stores nothing, and later batches keep the automatic rule."""
+    import paper_2107_09801_gb300 as P
+    cache = tmp_path / "tune.json"
+    with P.Context(arena_bytes=1 << 30, max_walks=400, max_sms=2) as ctx:
+        wid = ctx.submit_ex(70001, 1, 4, 13, 10)
+        assert ctx.hot_variant() == "k_lin + k_quad"
+        ctx.autotune(reps=1, cache=str(cache))
+        assert not cache.exists()
+        ctx.release(wid)
+        ctx.set_max_sms(0)
+        for q in range(400):
+            ctx.submit_ex(1023, q, 4, 13, 10)
+        assert ctx.hot_variant() == "k_hot_batched<512,16,4>"
+        assert ctx.autotune(reps=1, cache=str(cache)) and cache.exists()
