@@ -247,7 +247,7 @@ def kernels_per_step(breakdown: dict, kernel: str = "") -> int:
     """Kernel launches of one step from a per-phase breakdown of whole steps (a phase's
     launches count its brackets, one per step); `kernel` names the neighbourhood kernels."""
     steps = max(breakdown.get("hot", (0, 0.0))[0], 1)
-    per_phase = dict(KERNELS_PER_PHASE, hot=2 if kernel == "k_lin + k_quad" else 1)
+    per_phase = dict(KERNELS_PER_PHASE, hot=1 + kernel.count(" + "))
     total = sum(per_phase.get(k, 1) * n for k, (n, _) in breakdown.items() if n)
     return int(round(total / steps))
 

@@ -279,7 +279,9 @@ PSL_API int psl_autotune(psl_ctx *ctx, int reps);
 
 /* Writes into name (cap bytes, NUL-terminated, truncated if short) the name of the
  * neighbourhood kernel the next step of ctx launches, after admitting queued walks: e.g.
- * "k_hot_pc<28,32,8>", "k_hot_batched<512,16,4>", "k_hot_alpha2<256>", "k_hot_plain".
+ * "k_hot_pc<28,32,8>", "k_hot_batched<512,16,4>", "k_hot_alpha2<256>", "k_hot_plain", or
+ * "k_lin + k_quad" (the correlation form), after the table kernel's name and " + " when
+ * other walks of the batch are scored by the tables.
  * Returns the length of the full name, PSL_EINVAL for a null argument or cap < 1. */
 PSL_API int psl_hot_variant(psl_ctx *ctx, char *name, int32_t cap);
 

@@ -21,6 +21,7 @@
 // covers about (L-1)/32 words whatever its place in the sequence (the forward and backward
 // ranges add up to L - 1), so the warps of a block do equal work and no block waits on
 // another.
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 #include <cstdio>
@@ -341,7 +342,8 @@ cudaError_t launch_hot(const LaunchCtx &c) {
 int hot_kernel_name(const LaunchCtx &c, char *out, int cap) {
   if (c.alpha2) return snprintf(out, (size_t)cap, "k_hot_alpha2<%u>", c.hot_threads);
   if (c.lin && !c.tables) return snprintf(out, (size_t)cap, "k_lin + k_quad");
-  return hot_batched_name(c, out, cap);
+  const int n = hot_batched_name(c, out, cap);
+  return c.lin ? n + snprintf(out + std::min(n, cap - 1), (size_t)(cap - std::min(n, cap - 1)), " + k_lin + k_quad") : n;
 }
 
 }  // namespace psl

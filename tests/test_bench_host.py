@@ -90,3 +90,10 @@ def test_kernels_per_step():
     assert bench.kernels_per_step(general) == 7
     assert bench.kernels_per_step({"hot": (2, 1.0), "tail": (2, 0.1)}) == 2
     assert bench.kernels_per_step({"hot": (2, 1.0)}) == 1
+
+
+def test_kernels_per_step_counts_every_neighbourhood_kernel():
+    b = {"hot": (2, 1.0), "select": (2, 0.1), "recheck": (2, 0.1), "decide": (2, 0.1), "apply": (2, 0.1)}
+    assert bench.kernels_per_step(b, "k_hot_pc<28,32,8>") == 7
+    assert bench.kernels_per_step(b, "k_lin + k_quad") == 8
+    assert bench.kernels_per_step(b, "k_hot_batched<512,32,8> + k_lin + k_quad") == 9

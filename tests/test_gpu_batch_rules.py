@@ -62,3 +62,18 @@ def test_autotuner_leaves_the_choice_open_when_there_is_none(tmp_path):
             ctx.submit_ex(1023, q, 4, 13, 10)
         assert ctx.hot_variant() == "k_hot_batched<512,16,4>"
         assert ctx.autotune(reps=1, cache=str(cache)) and cache.exists()
+
+
+def test_kernel_name_of_a_mixed_batch():
+    import paper_2107_09801_gb300 as P
+    from paper_2107_09801_gb300 import binding as B
+    with P.Context(arena_bytes=1 << 30, max_walks=8, max_sms=2) as ctx:
+        for L in (1023, 40000, 70001):
+            ctx.submit_ex(L, L, 4, 13, 10)
+        full = ctx.hot_variant()
+        table, _, rest = full.partition(" + ")
+        assert table.startswith("k_hot_batched<") and rest == "k_lin + k_quad"
+        for cap in range(1, len(full) + 2):  # truncated like snprintf, NUL-terminated, the full length returned
+            buf = B.ct.create_string_buffer(b"x" * 63, 64)
+            assert B.lib().psl_hot_variant(ctx.h, buf, cap) == len(full)
+            assert buf.raw[:cap] == full.encode()[:cap - 1].ljust(cap, b"\0") and buf.raw[cap:cap + 1] == b"x"
