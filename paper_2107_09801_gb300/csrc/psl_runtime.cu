@@ -678,10 +678,13 @@ static int rebuild_active(psl_ctx *ctx) {
   for (uint32_t s : ctx->active)
     short_only = short_only && ctx->h_hdr[s].L <= kTailMaxL && ctx->h_hdr[s].N <= kTailMaxN &&
                  ctx->h_hdr[s].shard_count <= 1;
-  // One wave of eight-warp blocks (two fit an SM) is faster than one-warp blocks; more walks are not.
-  // Microseconds a step, one warp / eight: one walk of L = 1023 49.2 / 32.2, 304 of them 90.7 / 83.3, 608
-  // 139 / 145; 304 of L = 2047 157 / 139, of L = 300 53.5 / 52.8; one of L = 6000 (N = 2000) 127 / 40.
-  const bool wide = short_only && ctx->active.size() <= 2ull * ctx->sm_count;
+  // One wave of eight-warp blocks (two fit an SM) is faster than one-warp blocks; more walks are not, and
+  // several walks of one or two words are not, whose phases are more barriers than work.  Microseconds a step, one warp /
+  // eight: one walk of L = 1023 49.2 / 32.2, 304 of them 90.7 / 83.3, 608 139 / 145; 304 of L = 2047 157 / 139;
+  // one of L = 6000 (N = 2000) 127 / 40.  L = 31: 64 walks 28.3 / 29.1, 304 29.7 / 31.9; L = 63: 32.7 / 33.3, 34.0
+  // / 36.0; L = 100: 36.0 / 35.9, 39.5 / 40.7, but switching phase every few moves 66.8 / 58.9, 71.1 / 65.5.
+  const bool wide = short_only && ctx->active.size() <= 2ull * ctx->sm_count &&
+                    (ctx->active.size() == 1 || ctx->h_hdr[ctx->active[0]].L >= 64);  // the longest
   if (short_only != ctx->tail_fused || wide != ctx->tail_wide) {
     ctx->tail_fused = short_only;
     ctx->tail_wide = wide;
