@@ -77,3 +77,17 @@ def test_kernel_name_of_a_mixed_batch():
             buf = B.ct.create_string_buffer(b"x" * 63, 64)
             assert B.lib().psl_hot_variant(ctx.h, buf, cap) == len(full)
             assert buf.raw[:cap] == full.encode()[:cap - 1].ljust(cap, b"\0") and buf.raw[cap:cap + 1] == b"x"
+
+
+@pytest.mark.parametrize("L,walks,name", [(255, 152, "k_hot_batched<256,32,4>"), (128, 120, "k_hot_batched<256,32,4>"),
+                                          (255, 153, "k_hot_batched<512,16,4>"), (300, 114, "k_hot_batched<512,16,4>")])
+def test_walks_of_one_small_block_each(L, walks, name):
+    """On 152 SMs: blocks of 512 only when the blocks of 256 no longer have an SM each."""
+    import torch
+    import paper_2107_09801_gb300 as P
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the line depends on the number of SMs")
+    with P.Context(arena_bytes=walks * P.psl_walk_bytes(L, L, 0) + (64 << 20), max_walks=walks) as ctx:
+        for q in range(walks):
+            ctx.submit_ex(L, q, 4, 13, 10)
+        assert ctx.hot_variant() == name
