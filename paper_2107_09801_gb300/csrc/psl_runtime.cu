@@ -126,6 +126,21 @@ struct HostWalk {
 
 }  // namespace
 
+// What the nodes of a captured graph depend on.
+struct GraphKey {
+  LaunchCtx c{};
+  bool tail_fused = false;
+  uint32_t steps = 0;
+  bool operator==(const GraphKey &o) const {
+    return c.hdr == o.c.hdr && c.active == o.c.active && c.sched == o.c.sched && c.items == o.c.items &&
+           c.stream == o.c.stream && c.hot_threads == o.c.hot_threads && c.hot_tile_sb == o.c.hot_tile_sb &&
+           c.hot_flush_sb == o.c.hot_flush_sb && c.sm_count == o.c.sm_count && c.alpha2 == o.c.alpha2 &&
+           c.tail_wide == o.c.tail_wide && c.lin == o.c.lin && c.tables == o.c.tables && tail_fused == o.tail_fused &&
+           steps == o.steps;
+  }
+};
+constexpr size_t kKeptGraphs = 3;
+
 struct psl_ctx {
   psl_config cfg{};
   cudaStream_t stream = nullptr;
@@ -158,8 +173,12 @@ struct psl_ctx {
   uint32_t sm_count = 152;   // SMs the persistent kernels are sized for
   uint32_t dev_sms = 152;    // SMs of the device
   std::string err;
-  // CUDA graph of steps_per_graph steps over the current active set
+  // CUDA graph of steps_per_graph steps over the current active set, and those of other kernel choices that
+  // the batch has had (unprofiled ones, kKeptGraphs at most, the oldest first)
   cudaGraphExec_t graph = nullptr;
+  std::vector<GraphKey> kept_keys;
+  std::vector<cudaGraphExec_t> kept;
+  GraphKey graph_key;
   uint32_t graph_steps = 0;
   int graph_prof = 0;  // profile mode the graph was captured with (its event nodes)
   // CUDA-event profile of kernel launches: 0 off, 1 every kernel, 2 the neighbourhood kernel only
@@ -279,7 +298,44 @@ static void gprof_clear(psl_ctx *ctx) {
 static void drop_graph(psl_ctx *ctx) {
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
   ctx->graph = nullptr;
+  for (cudaGraphExec_t g : ctx->kept) cudaGraphExecDestroy(g);
+  ctx->kept.clear();
+  ctx->kept_keys.clear();
   gprof_clear(ctx);
+}
+
+// The batch takes other kernels: its graph is kept for when it takes these again.  (A context whose batch moves
+// around a line of the rules would capture on every crossing: 0.1 to 0.2 ms for 8 steps.)
+static void put_graph_by(psl_ctx *ctx) {
+  if (!ctx->graph) return;
+  if (ctx->graph_prof) {
+    cudaGraphExecDestroy(ctx->graph);  // its event pairs are the context's only ones
+    gprof_clear(ctx);
+  } else {
+    if (ctx->kept.size() == kKeptGraphs) {
+      cudaGraphExecDestroy(ctx->kept[0]);
+      ctx->kept.erase(ctx->kept.begin());
+      ctx->kept_keys.erase(ctx->kept_keys.begin());
+    }
+    ctx->kept.push_back(ctx->graph);
+    ctx->kept_keys.push_back(ctx->graph_key);
+  }
+  ctx->graph = nullptr;
+}
+
+// A kept graph of exactly these launches, taken out.
+static bool take_graph(psl_ctx *ctx, const GraphKey &key) {
+  for (size_t i = 0; i < ctx->kept.size(); i++)
+    if (ctx->kept_keys[i] == key) {
+      ctx->graph = ctx->kept[i];
+      ctx->graph_key = key;
+      ctx->graph_steps = key.steps;
+      ctx->graph_prof = 0;
+      ctx->kept.erase(ctx->kept.begin() + (ptrdiff_t)i);
+      ctx->kept_keys.erase(ctx->kept_keys.begin() + (ptrdiff_t)i);
+      return true;
+    }
+  return false;
 }
 
 // Folds the times of the last graph launch into the totals (the stream must be synchronised).
@@ -667,12 +723,12 @@ static int rebuild_active(psl_ctx *ctx) {
   if (any_lin != ctx->lin || any_tab != ctx->tables) {
     ctx->lin = any_lin;
     ctx->tables = any_tab;
-    drop_graph(ctx);  // captured with other kernels
+    put_graph_by(ctx);
   }
   const uint32_t fb = hot_flush_for(maxL);
   if (fb != ctx->hot_flush_sb) {
     ctx->hot_flush_sb = fb;
-    drop_graph(ctx);  // captured with the other kernel variant
+    put_graph_by(ctx);
   }
   bool short_only = !ctx->active.empty();
   for (uint32_t s : ctx->active)
@@ -688,7 +744,7 @@ static int rebuild_active(psl_ctx *ctx) {
   if (short_only != ctx->tail_fused || wide != ctx->tail_wide) {
     ctx->tail_fused = short_only;
     ctx->tail_wide = wide;
-    drop_graph(ctx);  // captured with the other kernel sequence
+    put_graph_by(ctx);
   }
   // alpha = 2 batches of short walks take the closed-form score (unless the configuration
   // asks for the tables); it scores every neighbour whole, so their k range is never split
@@ -699,7 +755,7 @@ static int rebuild_active(psl_ctx *ctx) {
   }
   if (a2 != ctx->alpha2) {
     ctx->alpha2 = a2;
-    drop_graph(ctx);  // captured with the other kernel
+    put_graph_by(ctx);
   }
   // Split every walk's k range into chunks when the neighbour blocks alone would leave
   // SMs idle (few walks, or a long walk on its own): aim for about four blocks per SM.
@@ -721,11 +777,11 @@ static int rebuild_active(psl_ctx *ctx) {
     if (t != ctx->cfg.hot_threads || sb != ctx->cfg.hot_tile_sb) {
       ctx->cfg.hot_threads = t;
       ctx->cfg.hot_tile_sb = sb;
-      drop_graph(ctx);  // captured with another kernel variant
+      put_graph_by(ctx);
     }
   } else if (ctx->hot_auto && (ctx->cfg.hot_threads != 256 || ctx->cfg.hot_tile_sb != 32)) {
     ctx->cfg.hot_threads = 256, ctx->cfg.hot_tile_sb = 32;
-    drop_graph(ctx);
+    put_graph_by(ctx);
   }
   const uint32_t T_tab = (uint32_t)ctx->cfg.hot_threads * (a2 ? kA2PerThread : 1u);  // window positions per item
   std::vector<HotItem> quad;
@@ -945,9 +1001,13 @@ static cudaError_t enqueue_batched_step(psl_ctx *ctx, const LaunchCtx &c, bool c
 // Captures steps_per_graph steps over the context's device schedule into one CUDA graph,
 // with event-record nodes around the kernels that the current profile mode times.
 static int capture_graph(psl_ctx *ctx) {
-  drop_graph(ctx);
+  if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+  ctx->graph = nullptr;
+  gprof_clear(ctx);
   const uint32_t G = (uint32_t)ctx->cfg.steps_per_graph;
   LaunchCtx c = launch_ctx(ctx, ctx->d_active, ctx->d_sched);
+  const GraphKey key{c, ctx->tail_fused, G};
+  if (!ctx->prof && take_graph(ctx, key)) return PSL_OK;
   if (ctx->prof) CK(gprof_reserve(ctx, (size_t)G * 5));  // at most five profiled phases a step
   cudaGraph_t g;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -965,6 +1025,7 @@ static int capture_graph(psl_ctx *ctx) {
     gprof_clear(ctx);
     return fail(ctx, PSL_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
   }
+  ctx->graph_key = key;
   ctx->graph_steps = G;
   ctx->graph_prof = ctx->prof;
   return PSL_OK;

@@ -91,3 +91,31 @@ def test_walks_of_one_small_block_each(L, walks, name):
         for q in range(walks):
             ctx.submit_ex(L, q, 4, 13, 10)
         assert ctx.hot_variant() == name
+
+
+@pytest.mark.parametrize("base,extra,sms", [([(1023, 4, 13)] * 16, (1023, 4, 13), 8), ([(511, 2, 2)] * 4, (300, 4, 13), 8),
+                                            ([(40000, 4, 13)] * 2, (1023, 4, 13), 2)])
+def test_batches_that_take_other_kernels_and_return(base, extra, sms):
+    """Graphs captured for one choice of kernels are used again when the batch returns to it."""
+    import paper_2107_09801_gb300 as P
+    spec = lambda q, t, budget: W.WalkSpec(L=t[0], seed=q, alpha1=t[1], alpha2=t[2], budget=budget, ls_lmt=3, n_lmt=6912)
+    got = []
+    for graph in (3, 0):
+        with P.Context(arena_bytes=1 << 30, max_walks=32, max_sms=sms, steps_per_graph=graph) as ctx:
+            specs = [spec(q, t, 33) for q, t in enumerate(base)]
+            ids = [submit_spec(ctx, s) for s in specs]
+            names, traces = set(), []
+            for r in range(5):
+                s = spec(100 + r, extra, 3)
+                wid = submit_spec(ctx, s)
+                names.add(ctx.hot_variant())
+                ctx.step(3)
+                traces.append(ctx.trace(wid, 3))
+                ctx.release(wid)
+                names.add(ctx.hot_variant())
+                ctx.step(3)
+            ctx.run()
+            got.append(traces + [ctx.trace(i, 33) for i in ids])
+    for tr, tr0 in zip(*got):
+        assert len(tr) and same_decisions(tr, tr0)
+    assert len(names) == 2 or base[0] == extra  # (there the step tail changes)
