@@ -229,14 +229,20 @@ def _code_only(src: str) -> str:
 
 
 def kernel_source_hash(kernel: str = "k_hot_batched") -> str:
-    """Hash of the code of a neighbourhood kernel (its translation unit and device header,
-    comments left out)."""
-    h = hashlib.sha256()
-    tu = ("psl_alpha2.cu" if kernel.startswith("k_hot_alpha2") else
-          "psl_lin.cu" if kernel.startswith("k_lin") else "psl_hot.cu")
-    for fn in (tu, "psl_device.cuh"):
-        with open(os.path.join(ROOT, "paper_2107_09801_gb300", "csrc", fn), encoding="utf-8") as f:
-            h.update(_code_only(f.read()).encode())
+    """Hash of the code of a neighbourhood kernel (its translation unit and the device headers
+    that it includes, directly or through one another; comments left out)."""
+    csrc = os.path.join(ROOT, "paper_2107_09801_gb300", "csrc")
+    todo = ["psl_alpha2.cu" if kernel.startswith("k_hot_alpha2") else
+            "psl_lin.cu" if kernel.startswith("k_lin") else "psl_hot.cu"]
+    h, seen = hashlib.sha256(), set(todo)
+    while todo:
+        with open(os.path.join(csrc, todo.pop(0)), encoding="utf-8") as f:
+            code = _code_only(f.read())
+        h.update(code.encode())
+        for fn in re.findall(r'#include "(\w+\.cuh)"', code):
+            if fn not in seen and os.path.exists(os.path.join(csrc, fn)):
+                seen.add(fn)
+                todo.append(fn)
     return h.hexdigest()[:16]
 
 

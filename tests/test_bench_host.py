@@ -97,3 +97,19 @@ def test_kernels_per_step_counts_every_neighbourhood_kernel():
     assert bench.kernels_per_step(b, "k_hot_pc<28,32,8>") == 7
     assert bench.kernels_per_step(b, "k_lin + k_quad") == 8
     assert bench.kernels_per_step(b, "k_hot_batched<512,32,8> + k_lin + k_quad") == 9
+
+
+@pytest.mark.parametrize("kernel,header,covered", [("k_hot_pc<28,32,8>", "psl_async.cuh", True), ("k_lin + k_quad", "psl_async.cuh", True),
+                                                   ("k_lin + k_quad", "psl_device.cuh", True), ("k_hot_alpha2<256>", "psl_async.cuh", False)])
+def test_kernel_hash_covers_the_headers_it_includes(tmp_path, monkeypatch, kernel, header, covered):
+    csrc = tmp_path / "paper_2107_09801_gb300" / "csrc"
+    shutil.copytree(os.path.join(bench.ROOT, "paper_2107_09801_gb300", "csrc"), csrc)
+    before = bench.kernel_source_hash(kernel)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.kernel_source_hash(kernel) == before
+    with open(csrc / header, "a") as f:
+        f.write("// a remark\n")
+    assert bench.kernel_source_hash(kernel) == before
+    with open(csrc / header, "a") as f:
+        f.write("static int unused_probe_value;\n")
+    assert (bench.kernel_source_hash(kernel) != before) == covered
