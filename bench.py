@@ -339,6 +339,14 @@ def term_counts(L: int) -> dict:
             "lookups": float((2.0 * kin / 5.0 + (kout - kin) / 5.0).mean()), "quad": float((kin / 5.0).mean())}
 
 
+def tensor_peak():
+    """(bf16 FLOP/s of a library GEMM on this GPU model, where the figure comes from)."""
+    try:
+        return json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["bf16_tflops"] * 1e12, "measured bf16 GEMM"
+    except Exception:
+        return 1.9e15, "bf16 GEMM, an earlier measurement on a GB300"
+
+
 def measure_alu_peak(local: int, stream) -> dict:
     """The microbenchmarks of the CUDA-core pipes (psl_alu_peak) with the SM clock sampled
     while they run."""
@@ -354,10 +362,10 @@ def hot_roofline(walks_x_N: int, L: int, hot_avg_ms: float, peak: dict, mhz_run:
                  kernel: str, psls=()) -> dict:
     """Roofline of the neighbourhood kernel: 2 lane-ops per (neighbour, shift) term against the
     measured FP32-add / integer-add / logic-op mix rate, scaled to the clock of the timed region;
-    also on live terms, and against the lookup ceiling of the kernel's own inner pattern."""
+    also on live terms, and against the lookup ceiling of the kernel's own inner pattern.  The
+    correlation form's two kernels run one after the other, the first bound by the tensor cores and
+    the second by lookups: its peak is the rate at which both would run at their own ceilings."""
     tc = term_counts(L)
-    if kernel == "k_lin + k_quad":
-        tc["lookups"] = tc["quad"]
     mhz_peak = peak["clocks"].get("sm_mhz") or peak["max_clock_mhz"]
     scale = (mhz_run / mhz_peak) if (mhz_run and mhz_peak) else 1.0
     p_mix = peak["mix"] * scale
@@ -365,20 +373,36 @@ def hot_roofline(walks_x_N: int, L: int, hot_avg_ms: float, peak: dict, mhz_run:
     sec = hot_avg_ms / 1000.0
     achieved = walks_x_N * 2 * tc["nominal"] / sec
     achieved_live = walks_x_N * 2 * tc["live"] / sec
-    lookups = walks_x_N * tc["lookups"] / sec
-    out = {"bound": "alu", "kernel": kernel, "achieved": achieved / 1e12, "peak": p_mix / 1e12,
-           "unit": "Tops/s", "frac": achieved / p_mix,
-           "peak_basis": f"measured: psl_alu_peak mix microbenchmark (FP32 add, integer add, logic op 1:1:1 on "
-                         f"{peak['sm_count']} SMs) {peak['mix'] / 1e12:.2f} Tops/s at {mhz_peak:.0f} MHz, scaled to "
-                         f"the timed region's {mhz_run:.0f} MHz",
-           "ops_basis": "2 lane-ops per (neighbour, shift) term, (L-1) terms per flip-eval",
-           "frac_live_terms": achieved_live / p_mix,
-           "live_basis": f"2 lane-ops per term with a partner: {tc['live']:.0f} of {tc['nominal']:.0f} shifts per "
-                         "flip-eval on average",
-           "lookup_ceiling": {"lookups_per_s_measured": peak["lookup"], "lookups_per_flip_eval": tc["lookups"],
-                              "flip_evals_per_s_ceiling": p_lookup / tc["lookups"],
-                              "frac": lookups / p_lookup},
-           "traffic": None, "issue_frac": None}
+    if kernel == "k_lin + k_quad":
+        tensor, basis = tensor_peak()
+        flops = 2 * 3 * tc["nominal"]  # three digits of each coefficient times every partner's +-1
+        t_tensor, t_lookup = walks_x_N * flops / tensor, walks_x_N * tc["quad"] / p_lookup
+        peak_rate = walks_x_N / (t_tensor + t_lookup)
+        out = {"bound": "tensor+lookups", "kernel": kernel, "achieved": walks_x_N / sec, "peak": peak_rate,
+               "unit": UNIT, "frac": walks_x_N / sec / peak_rate,
+               "peak_basis": f"k_lin at {tensor / 1e12:.0f} TFLOP/s ({basis}), then k_quad at the lookup "
+                             f"microbenchmark's {peak['lookup'] / 1e12:.2f} T/s at {mhz_peak:.0f} MHz, scaled to the "
+                             f"timed region's {mhz_run:.0f} MHz",
+               "ops_basis": f"per flip-eval {flops:.0f} tensor FLOP (partners outside the sequence and chunks done "
+                             f"twice not counted) and {tc['quad']:.0f} lookups",
+               "tensor_ms": 1e3 * t_tensor, "lookup_ms": 1e3 * t_lookup, "frac_live_terms": None,
+               "lookup_ceiling": None, "frac_nominal_terms_of_alu_mix": achieved / p_mix,
+               "traffic": None, "issue_frac": None}
+    else:
+        lookups = walks_x_N * tc["lookups"] / sec
+        out = {"bound": "alu", "kernel": kernel, "achieved": achieved / 1e12, "peak": p_mix / 1e12,
+               "unit": "Tops/s", "frac": achieved / p_mix,
+               "peak_basis": f"measured: psl_alu_peak mix microbenchmark (FP32 add, integer add, logic op 1:1:1 on "
+                             f"{peak['sm_count']} SMs) {peak['mix'] / 1e12:.2f} Tops/s at {mhz_peak:.0f} MHz, scaled to "
+                             f"the timed region's {mhz_run:.0f} MHz",
+               "ops_basis": "2 lane-ops per (neighbour, shift) term, (L-1) terms per flip-eval",
+               "frac_live_terms": achieved_live / p_mix,
+               "live_basis": f"2 lane-ops per term with a partner: {tc['live']:.0f} of {tc['nominal']:.0f} shifts per "
+                             "flip-eval on average",
+               "lookup_ceiling": {"lookups_per_s_measured": peak["lookup"], "lookups_per_flip_eval": tc["lookups"],
+                                  "flip_evals_per_s_ceiling": p_lookup / tc["lookups"],
+                                  "frac": lookups / p_lookup},
+               "traffic": None, "issue_frac": None}
     if kernel.startswith("k_hot_alpha2"):
         # the closed form does no table lookups: its own ceiling is the bit-plane step rate
         steps = plane_steps_per_flip_eval(L, psls)

@@ -113,3 +113,19 @@ def test_kernel_hash_covers_the_headers_it_includes(tmp_path, monkeypatch, kerne
     with open(csrc / header, "a") as f:
         f.write("static int unused_probe_value;\n")
     assert (bench.kernel_source_hash(kernel) != before) == covered
+
+
+def test_hot_roofline_correlation_form(monkeypatch):
+    """Two kernels one after the other: the ceiling is that of both at their own rates, and 1 is not exceeded by
+    a time that neither could reach."""
+    monkeypatch.setattr(bench, "tensor_peak", lambda: (2e15, "test"))
+    L, wn = 131071, 1024 * 6912
+    t_tensor = wn * 6 * (L - 1) / 2e15
+    t_lookup = wn * bench.term_counts(L)["quad"] / 4e12  # 8e12 at 2000 MHz, run at 1000
+    for ms in (16.1, 1e3 * (t_tensor + t_lookup)):
+        r = bench.hot_roofline(wn, L, ms, _peak(), 1000.0, None, "k_lin + k_quad")
+        assert r["bound"] == "tensor+lookups" and r["kernel"] == "k_lin + k_quad"
+        assert r["frac"] == pytest.approx((t_tensor + t_lookup) * 1e3 / ms)
+        assert r["achieved"] / r["peak"] == pytest.approx(r["frac"])
+        assert (r["tensor_ms"], r["lookup_ms"]) == pytest.approx((1e3 * t_tensor, 1e3 * t_lookup))
+        assert r["lookup_ceiling"] is None and r["frac_live_terms"] is None
