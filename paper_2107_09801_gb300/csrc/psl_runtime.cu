@@ -772,7 +772,28 @@ static int rebuild_active(psl_ctx *ctx) {
     for (uint32_t s : ctx->active)
       if (!ctx->h_hdr[s].lin && ctx->h_hdr[s].shard_count <= 1)
         b512 += (ctx->h_hdr[s].N + 511) / 512, b256 += (ctx->h_hdr[s].N + 255) / 256;
-    const bool big = fb == 4 ? 4 * b512 >= 3ull * ctx->sm_count && b256 > ctx->sm_count : b512 >= 4ull * ctx->sm_count;
+    bool big = fb == 4 ? 4 * b512 >= 3ull * ctx->sm_count && b256 > ctx->sm_count : b512 >= 4ull * ctx->sm_count;
+    if (big && fb != 4) {
+      // a few long walks among many short ones: their blocks are the last to finish, and blocks of 256 spread
+      // them over more SMs.  Microseconds of a batch: its blocks' own time over the SMs, and that of a longest
+      // block where those leave SMs idle.  Fitted to 90 batches of one to 50 walks of L = 8191 to 131071 among 100
+      // to 3000 of L = 300 to 4093, of which it takes the slower form by more than 1.5% in three (by 5% at most).
+      // 256/32 against 512/32: 300 of L = 1023 and one of L = 131071 549 / 845, 3000 and 16 1879 / 1678; 700 of
+      // L = 300 and one of L = 16383 174 / 194, 2000 and one 349 / 272.
+      auto cost = [&](uint32_t threads, double fixed, double per_shift, double alone) {
+        double sum = 0.0, longest = 0.0, blocks = 0.0;  // active: longest first
+        for (uint32_t s : ctx->active) {
+          const WalkDev &h = ctx->h_hdr[s];
+          if (h.lin || h.shard_count > 1) continue;
+          const double b = (h.N + threads - 1) / threads;
+          longest = std::max(longest, (double)h.L);
+          if (2.0 * h.L >= longest) blocks += b;
+          sum += b * (fixed + per_shift * h.L);
+        }
+        return sum / ctx->sm_count + alone * longest * std::max(0.0, 1.0 - blocks / (2.0 * ctx->sm_count));
+      };
+      big = cost(512, 10.0, 2.4e-3, 4.5e-3) < cost(256, 6.7, 1.44e-3, 3.0e-3);
+    }
     const int32_t t = big ? 512 : 256, sb = big && fb == 4 ? 16 : 32;
     if (t != ctx->cfg.hot_threads || sb != ctx->cfg.hot_tile_sb) {
       ctx->cfg.hot_threads = t;

@@ -119,3 +119,21 @@ def test_batches_that_take_other_kernels_and_return(base, extra, sms):
     for tr, tr0 in zip(*got):
         assert len(tr) and same_decisions(tr, tr0)
     assert len(names) == 2 or base[0] == extra  # (there the step tail changes)
+
+
+@pytest.mark.parametrize("batch,name", [([(131071, 1), (1023, 310)], "k_hot_batched<256,32,8>"),
+                                        ([(16383, 1), (1023, 310)], "k_hot_batched<256,32,8>"),
+                                        ([(16383, 1), (300, 2000)], "k_hot_batched<512,32,8>"),
+                                        ([(8191, 50), (1023, 310)], "k_hot_batched<512,32,8>")])
+def test_few_long_walks_among_short_ones(batch, name):
+    """On 152 SMs: the long walks' blocks finish last, and blocks of 256 spread them over more SMs."""
+    import torch
+    import paper_2107_09801_gb300 as P
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the line depends on the number of SMs")
+    need = sum(n * P.psl_walk_bytes(L, 6912, 0) for L, n in batch)
+    with P.Context(arena_bytes=need + (64 << 20), max_walks=sum(n for _, n in batch)) as ctx:
+        for L, n in batch:
+            for q in range(n):
+                ctx.submit_ex(L, q, 4, 13, 10)
+        assert ctx.hot_variant() == name
