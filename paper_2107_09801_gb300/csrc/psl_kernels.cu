@@ -52,12 +52,12 @@ __global__ void k_init_bits(WalkDev *hdr, const uint32_t *active) {
   if (idx == 0) W.psl = 0;
 }
 
-// Bits (1 for a negative value) of nseq +-1 sequences of L bytes, one warp a word.
-__global__ void __launch_bounds__(256) k_pack_pm1(const int8_t *__restrict__ seq, uint32_t L, uint32_t nw, WalkDev *hdr) {
-  const uint32_t i = blockIdx.x * 256u + threadIdx.x;
-  const bool neg = i < L && seq[(size_t)blockIdx.y * L + i] < 0;
+// Bits (1 for a negative value) of nseq +-1 sequences of L bytes with their zero guard words, one warp a word.
+__global__ void __launch_bounds__(256) k_pack_pm1(const int8_t *__restrict__ seq, int L, int nw, WalkDev *hdr) {
+  const int i = (int)(blockIdx.x * 256u + threadIdx.x) - 32 * kGuardWords, w = i >> 5;
+  const bool neg = i >= 0 && i < L && seq[(size_t)blockIdx.y * (size_t)L + (size_t)i] < 0;
   const uint32_t word = __ballot_sync(0xffffffffu, neg);
-  if ((threadIdx.x & 31) == 0 && (i >> 5) < nw) hdr[blockIdx.y].bits[i >> 5] = word;
+  if ((threadIdx.x & 31) == 0 && w < nw + kGuardWords) hdr[blockIdx.y].bits[w] = word;
 }
 
 // C_k = (L-k) - 2 popc(x[0..L-k) xor x[k..L)) for one k per thread (Eq. 2 on packed bits);
@@ -196,7 +196,8 @@ cudaError_t launch_init_bits(const LaunchCtx &c) {
 }
 
 cudaError_t launch_pack_pm1(const LaunchCtx &c, const int8_t *seq) {
-  k_pack_pm1<<<dim3((c.maxL + 255) / 256, c.ninit), 256, 0, c.stream>>>(seq, c.maxL, (c.maxL + 31) / 32, c.hdr);
+  const uint32_t nw = (c.maxL + 31) / 32, bits = 32 * (nw + 2 * kGuardWords);
+  k_pack_pm1<<<dim3((bits + 255) / 256, c.ninit), 256, 0, c.stream>>>(seq, (int)c.maxL, (int)nw, c.hdr);
   return cudaGetLastError();
 }
 

@@ -1456,10 +1456,10 @@ extern "C" int psl_autocorr(psl_ctx *ctx, const int8_t *seq, uint32_t nseq, uint
   // runs as init-only walks in temporary slots of a private header array
   const uint32_t nw = (L + 31) / 32;
   const size_t words = nw + 2 * kGuardWords;
-  // Three bit arrays a sequence, then every C, copied back at once.  The sequences go in as they came, where C
+  // The bits of every sequence, then every C, copied back at once.  The sequences go in as they came, where C
   // will be, and are packed on the device: with packing on the host and two copies a sequence the call took
   // 7.2 ms at 32 sequences of L = 65535, now 0.9.
-  const size_t per = align_up(words * 4, 256) * 3, c_bytes = (size_t)nseq * L * 4;
+  const size_t per = align_up(words * 4, 256), c_bytes = (size_t)nseq * L * 4;
   char *buf = nullptr;
   WalkDev *dh = nullptr;
   uint32_t *dl = nullptr;
@@ -1472,13 +1472,9 @@ extern "C" int psl_autocorr(psl_ctx *ctx, const int8_t *seq, uint32_t nseq, uint
   for (uint32_t q = 0; q < nseq; q++) {
     WalkDev &h = hh[q];
     std::memset(&h, 0, sizeof h);
-    char *b = buf + per * q;
     h.L = L;
     h.nw = nw;
-    h.has_init_seq = 1;
-    h.bits = (uint32_t *)b + kGuardWords;
-    h.bits_local = (uint32_t *)(b + align_up(words * 4, 256)) + kGuardWords;
-    h.bits_best = (uint32_t *)(b + 2 * align_up(words * 4, 256)) + kGuardWords;
+    h.bits = (uint32_t *)(buf + per * q) + kGuardWords;
     h.C = d_C + (size_t)q * L;
     h.status = kRunning;
     list[q] = q;
@@ -1496,8 +1492,7 @@ extern "C" int psl_autocorr(psl_ctx *ctx, const int8_t *seq, uint32_t nseq, uint
     c.ninit = nseq;
     c.sm_count = ctx->sm_count;
     c.stream = ctx->stream;
-    e = launch_init_bits(c);
-    if (e == cudaSuccess) e = launch_pack_pm1(c, d_seq);
+    e = launch_pack_pm1(c, d_seq);
     if (e == cudaSuccess) e = launch_autocorr(c);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(C, d_C, c_bytes, cudaMemcpyDeviceToHost, ctx->stream);
