@@ -765,14 +765,18 @@ static int rebuild_active(psl_ctx *ctx) {
   // fill more SMs with blocks of 256.  Microseconds a step, 256/32 against the choice here: 4096 walks of
   // L = 1023 1692 / 718 (512/16), 64 of them 77.7 / 64.1, 256 of L = 4093 537 / 317, 2048 of L = 300
   // 643 / 221; 64 of L = 8191 264 / 225 (512/32), 32 of them 160 / 164 and 64 of L = 300 49.0 / 52.2, so
-  // those keep 256/32; so do walks of one block of 256 while every block has an SM (152 of L = 255 48.5 / 51.3,
-  // 153 of them 58.7 / 52.0).
+  // those keep 256/32; so do batches of walks of one block of 256 while every block has an SM (152 of L = 255
+  // 48.5 / 51.3, 153 of them 58.7 / 52.0; with four of L = 2047 among 120 of L = 255 73.8 / 55.5).
   if (ctx->hot_auto && !a2) {
-    uint64_t b512 = 0, b256 = 0;
+    uint64_t b512 = 0;
+    uint32_t maxN = 0;
     for (uint32_t s : ctx->active)
-      if (!ctx->h_hdr[s].lin && ctx->h_hdr[s].shard_count <= 1)
-        b512 += (ctx->h_hdr[s].N + 511) / 512, b256 += (ctx->h_hdr[s].N + 255) / 256;
-    bool big = fb == 4 ? 4 * b512 >= 3ull * ctx->sm_count && b256 > ctx->sm_count : b512 >= 4ull * ctx->sm_count;
+      if (!ctx->h_hdr[s].lin && ctx->h_hdr[s].shard_count <= 1) {
+        b512 += (ctx->h_hdr[s].N + 511) / 512;
+        maxN = std::max(maxN, ctx->h_hdr[s].N);
+      }
+    bool big = fb == 4 ? (maxN <= 256 ? b512 > ctx->sm_count : 4 * b512 >= 3ull * ctx->sm_count)
+                       : b512 >= 4ull * ctx->sm_count;
     if (big && fb != 4) {
       // a few long walks among many short ones: their blocks are the last to finish, and blocks of 256 spread
       // them over more SMs.  Microseconds of a batch: its blocks' own time over the SMs, and that of a longest

@@ -124,7 +124,8 @@ def test_batches_that_take_other_kernels_and_return(base, extra, sms):
 @pytest.mark.parametrize("batch,name", [([(131071, 1), (1023, 310)], "k_hot_batched<256,32,8>"),
                                         ([(16383, 1), (1023, 310)], "k_hot_batched<256,32,8>"),
                                         ([(16383, 1), (300, 2000)], "k_hot_batched<512,32,8>"),
-                                        ([(8191, 50), (1023, 310)], "k_hot_batched<512,32,8>")])
+                                        ([(8191, 50), (1023, 310)], "k_hot_batched<512,32,8>"),
+                                        ([(2047, 4), (255, 120)], "k_hot_batched<512,16,4>")])
 def test_few_long_walks_among_short_ones(batch, name):
     """On 152 SMs: the long walks' blocks finish last, and blocks of 256 spread them over more SMs."""
     import torch
