@@ -5,7 +5,8 @@
 // One walk step (the body of the while loop of Algorithm 1) is five phases:
 //   hot     FP32 filter score of every neighbour in the window (Eq. 4 through the
 //           one-element flip of Sec. 3) and, when it can matter, its exact PSL (Eq. 3)
-//           -- psl_hot.cu (subset-sum tables), psl_alpha2.cu (the closed form at alpha = 2)
+//           -- psl_hot.cu (subset-sum tables), psl_lin.cu (batches of long walks: a correlation on the
+//           tensor cores and one table a group), psl_alpha2.cu (the closed form at alpha = 2)
 //   select  minimum score, the certified candidate set {score <= min + 2B} plus the
 //           FP32 top-k, and the first neighbour of minimum PSL
 //   recheck exact Delta F of every candidate -- psl_recheck.cu (two kernels)

@@ -17,7 +17,8 @@
 // p = jA + 64 (b + tau) + x, x < 64.  For one chunk tau,
 //   Y[b, a] += sum_x S[b + tau, x] G[64 tau + x - a],   S[r, x] = s_{jA + 64 r + x} (0 outside),
 // is a 128 x 64 x 64 product: tcgen05.mma kind::f16, M = 128, N = 192, four steps of K = 16.
-//   * G in fixed point: B_k and D_k are rounded once to multiples of 2^-lin_sh (35 bits) and split
+//   * G in fixed point: B_k and D_k are rounded once to multiples of 2^-lin_sh (35 bits for the largest; a
+//     coefficient 2^-11 of it keeps as many as FP32, smaller ones fewer, the least round to zero) and split
 //     into three balanced base-4096 digits, each exact in f16; the digits are the three column
 //     groups of N.  Sums of at most 8192 products of +-1 with |digit| <= 2048 stay within 2^24, so
 //     the FP32 accumulators hold exact integers; every 128 chunks they are added into 64-bit
@@ -40,10 +41,10 @@
 // agree on which items exist.
 //
 // What bounds it, at 304 walks of L = 131071 (N = 6912; two or three tiles per SM): k_lin 2.3 ms, the
-// tensor pipe active 57% of it (386 cycles a chunk; the rest is the issuing threads' instruction latency, the
-// chunks done twice and the readings of the accumulators); k_quad 2.9 ms, 77% of the issue slots and 57% of
-// the shared-memory wavefronts (two ALU instructions and one lookup per five shifts).  The tables alone took
-// 11.2 ms.  A whole step of 1024 such walks: 38.3 -> 21.2 ms.
+// tensor pipe active 58% of it (386 cycles a chunk; the rest is the issuing threads' instruction latency, the
+// chunks done twice and the readings of the accumulators); k_quad 2.9 ms, 77% of the issue slots, 71% of the ALU
+// pipe and 57% of the shared-memory wavefronts (two ALU instructions and one lookup per five shifts).  The
+// tables alone took 10.1 ms.  A whole step of 1024 such walks: 35.2 -> 17.9 ms.
 #include <climits>
 #include <cstdint>
 #include <cstdio>

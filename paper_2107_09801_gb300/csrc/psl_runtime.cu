@@ -757,8 +757,6 @@ static int rebuild_active(psl_ctx *ctx) {
     ctx->alpha2 = a2;
     put_graph_by(ctx);
   }
-  // Split every walk's k range into chunks when the neighbour blocks alone would leave
-  // SMs idle (few walks, or a long walk on its own): aim for about four blocks per SM.
   // Block and tile of the table kernel when the configuration leaves them open.  Blocks of 512 share each
   // table between twice the neighbours, and a tile of 16 lets two of them fit an SM with the short
   // walks' five tables a group, where one block of 256 with a tile of 32 is all that fits; a few walks
@@ -808,6 +806,8 @@ static int rebuild_active(psl_ctx *ctx) {
     ctx->cfg.hot_threads = 256, ctx->cfg.hot_tile_sb = 32;
     put_graph_by(ctx);
   }
+  // Split every walk's k range into chunks when the neighbour blocks alone would leave
+  // SMs idle (few walks, or a long walk on its own): aim for about four blocks per SM.
   const uint32_t T_tab = (uint32_t)ctx->cfg.hot_threads * (a2 ? kA2PerThread : 1u);  // window positions per item
   std::vector<HotItem> quad;
   uint64_t nblocks = 0;
